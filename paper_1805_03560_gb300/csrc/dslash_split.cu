@@ -1,0 +1,304 @@
+// Hemi-Dslash with one thread per site and direction, for lattices too small
+// to fill the GPU with one thread per site (the operator and its algebra:
+// dslash.cu).
+//
+// A block takes 32 consecutive sites and four warps; warp mu holds the two
+// hops of direction mu of every site.  Each thread loads both neighbour
+// spinors and both links at once, accumulates the two hops, and leaves the
+// twelve components in shared memory; after one barrier the warps add the
+// four directions of each output component and run the epilogue on one
+// 16-byte chunk per thread.
+//
+// What bounds the small lattices is latency: one thread per site waits for
+// eight hops' loads one after another, on a GPU mostly empty (8^3 x 16: 32
+// blocks of 128 threads on 152 SMs).  Here a site's loads are all in flight,
+// every SM has work from 4864 sites on, and inside a solve the loads of the
+// links, which none of its launches writes, are issued before the wait for
+// the launch before (links_ready).  Measured (one thread per site -> this
+// kernel): a CG iteration in FP32 on 8^3 x 16 33.1 -> 23.2 us, on 14 x 6 x 10
+// x 20 33.7 -> 24.8 us, on 12^3 x 24 36.8 -> 30.8 us; in FP64 155 -> 84, 201 ->
+// 131 and 282 -> 208 us; the emulated-FP64 hop 22.0 -> 9.7, 22.8 -> 10.8 and 30.4
+// -> 18.2 us.  (One thread per hop, eight warps to 32 sites, was slower for
+// FP32: 38.6 us per iteration on 12^3 x 24, the barrier's traffic doubles.)
+#include "dslash_ops.cuh"
+#include "hmc_host.h"
+
+namespace hmc {
+
+namespace {
+
+constexpr int SPLIT_SITES = 32;
+constexpr int SPLIT_NT = 4 * SPLIT_SITES;
+
+// 16-byte chunk c of element s: CPC complex components per chunk
+template <int P>
+struct ChunkIO;
+template <>
+struct ChunkIO<HMC_F32> {
+  using R = float;
+  static constexpr int CPC = 2;
+  static __device__ __forceinline__ void load(const void *b, int S, int c, int s, Cx<float> v[2]) {
+    const float4 t = *((const float4 *)b + f32_chunk<6>(S, c, s));
+    v[0] = {t.x, t.y};
+    v[1] = {t.z, t.w};
+  }
+  static __device__ __forceinline__ void store(void *b, int S, int c, int s, const Cx<float> v[2]) {
+    *((float4 *)b + f32_chunk<6>(S, c, s)) = make_float4(v[0].re, v[0].im, v[1].re, v[1].im);
+  }
+};
+template <>
+struct ChunkIO<HMC_F64> {
+  using R = double;
+  static constexpr int CPC = 1;
+  static __device__ __forceinline__ void load(const void *b, int S, int c, int s, Cx<double> v[1]) {
+    const double2 t = *((const double2 *)b + (size_t)c * S + s);
+    v[0] = {t.x, t.y};
+  }
+  static __device__ __forceinline__ void store(void *b, int S, int c, int s, const Cx<double> v[1]) {
+    *((double2 *)b + (size_t)c * S + s) = make_double2(v[0].re, v[0].im);
+  }
+};
+template <>
+struct ChunkIO<HMC_F64E> {
+  using R = df64;
+  static constexpr int CPC = 1;
+  static __device__ __forceinline__ void load(const void *b, int S, int c, int s, Cx<df64> v[1]) {
+    const float4 t = *((const float4 *)b + (size_t)c * S + s);
+    v[0] = {df64(t.x, t.y), df64(t.z, t.w)};
+  }
+  static __device__ __forceinline__ void store(void *b, int S, int c, int s, const Cx<df64> v[1]) {
+    *((float4 *)b + (size_t)c * S + s) = make_float4(v[0].re.hi, v[0].re.lo, v[0].im.hi,
+                                                     v[0].im.lo);
+  }
+};
+
+// project and accumulate of a direction known at run time (uniform over a warp)
+template <int S, typename R>
+__device__ __forceinline__ void project_mu(int mu, const Cx<R> p[12], Cx<R> h[6]) {
+  switch (mu) {
+    case 0: project<0, S>(p, h); break;
+    case 1: project<1, S>(p, h); break;
+    case 2: project<2, S>(p, h); break;
+    default: project<3, S>(p, h); break;
+  }
+}
+template <int S, typename R>
+__device__ __forceinline__ void accumulate_mu(int mu, Cx<R> acc[12], const Cx<R> w[6]) {
+  switch (mu) {
+    case 0: accumulate<0, S>(acc, w); break;
+    case 1: accumulate<1, S>(acc, w); break;
+    case 2: accumulate<2, S>(acc, w); break;
+    default: accumulate<3, S>(acc, w); break;
+  }
+}
+
+// fermion boundary sign of a hop in time that wraps around
+template <typename R>
+__device__ __forceinline__ void flip(bool wrap, Cx<R> h[6]) {
+  if (wrap) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) h[k] = -h[k];
+  }
+}
+
+template <int SP>
+constexpr int split_min_blocks() {
+  return SP == HMC_F32 ? 5 : 3;
+}
+
+template <int SP, int FMT, bool DAG>
+__global__ void __launch_bounds__(SPLIT_NT, split_min_blocks<SP>()) k_dslash_split(
+    const DslashArgs a) {
+  using SIO = SpinorIO<SP>;
+  using R = typename SIO::R;
+  using LIO = LinkIO<SP, FMT>;
+  using CIO = ChunkIO<SP>;
+  constexpr int SF = DAG ? -1 : 1;
+  constexpr int CPC = CIO::CPC, NCH = 12 / CPC;
+  __shared__ __align__(16) Cx<R> s_w[4][NCH][SPLIT_SITES][CPC];
+  __shared__ R s_n[4][SPLIT_SITES];
+  griddep_launch_dependents();
+  const int mu = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int Vh = a.g.Vh;
+  const int i = blockIdx.x * SPLIT_SITES + lane;
+  const bool in = i < Vh;
+  const int is = in ? i : Vh - 1;  // threads past the end work on the last site and store nothing
+  int c[4];
+  const int lex = site_coords(a.g, is, a.p, c);
+  const int cm = mu == 0 ? c[0] : mu == 1 ? c[1] : mu == 2 ? c[2] : c[3];
+  const int Lm = a.g.L[mu], stm = a.g.st[mu];
+  const int hf = (lex + (cm + 1 == Lm ? 1 - Lm : 1) * stm) >> 1;
+  const int hb = (lex + (cm == 0 ? Lm - 1 : -1) * stm) >> 1;
+  const bool wf = mu == 0 && cm + 1 == Lm, wb = mu == 0 && cm == 0;
+  const void *gf = link_base<SP, FMT>(a.gauge, Vh, a.p, mu);
+  const void *gb = link_base<SP, FMT>(a.gauge, Vh, 1 - a.p, mu);
+  Cx<R> acc[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) acc[k] = {R(0), R(0)};
+  if constexpr (SP == HMC_F64E) {
+    griddep_wait();
+    if (a.gate && *a.gate == 0) return;
+#pragma unroll 1
+    for (int d = 0; d < 2; ++d) {
+      Cx<R> psi[12], u[9], hs[6], w[6];
+      SIO::load(a.in, Vh, d ? hb : hf, psi);
+      LIO::load(d ? gb : gf, Vh, d ? hb : is, u);
+      const int S = d ? -SF : SF;
+      project_rt(mu, S, psi, hs);
+      flip(d ? wb : wf, hs);
+      if (d)
+        mul_link_dag(u, hs, w);
+      else
+        mul_link(u, hs, w);
+      accumulate_rt(mu, S, acc, w);
+    }
+  } else {
+    Cx<R> uf[9], ub[9], pf[12], pb[12], hs[6], w[6];
+    if (!a.links_ready) griddep_wait();
+    LIO::load(gf, Vh, is, uf);
+    LIO::load(gb, Vh, hb, ub);
+    if (a.links_ready) griddep_wait();
+    if (a.gate && *a.gate == 0) return;
+    SIO::load(a.in, Vh, hf, pf);
+    SIO::load(a.in, Vh, hb, pb);
+    project_mu<SF>(mu, pf, hs);
+    flip(wf, hs);
+    mul_link(uf, hs, w);
+    accumulate_mu<SF>(mu, acc, w);
+    project_mu<-SF>(mu, pb, hs);
+    flip(wb, hs);
+    mul_link_dag(ub, hs, w);
+    accumulate_mu<-SF>(mu, acc, w);
+  }
+  if (a.red_src && blockIdx.x == 0) {
+    const double t = block_sum_partials<SPLIT_NT>(a.red_src, a.red_n);
+    if (threadIdx.x == 0) {
+      *a.red_dst = t;
+      if (a.red_alpha) {
+        const double al = *a.red_rr / t;
+        *a.red_alpha = al;
+        if (!isfinite(al) || !(t > 0.0)) *a.red_flag = 2;
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < NCH; ++k)
+#pragma unroll
+    for (int j = 0; j < CPC; ++j) s_w[mu][k][lane][j] = acc[k * CPC + j];
+  __syncthreads();
+  R n2 = R(0);
+  if (in) {
+    const R cb = (R)a.cb, ca = (R)a.ca;
+    const R alpha = a.cg_x ? (R)*a.cg_alpha : R(0);
+#pragma unroll
+    for (int ch = mu; ch < NCH; ch += 4) {
+      Cx<R> t[CPC], v[CPC];
+#pragma unroll
+      for (int j = 0; j < CPC; ++j)
+        t[j] = ((s_w[0][ch][lane][j] + s_w[1][ch][lane][j]) + s_w[2][ch][lane][j]) +
+               s_w[3][ch][lane][j];
+      if (a.x) {
+        CIO::load(a.x, Vh, ch, i, v);
+#pragma unroll
+        for (int j = 0; j < CPC; ++j) {
+          t[j].re = fma(ca, v[j].re, cb * t[j].re);
+          t[j].im = fma(ca, v[j].im, cb * t[j].im);
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < CPC; ++j) t[j] = cb * t[j];
+      }
+      if (a.cg_x) {
+        // fused CG step: x += alpha p, r -= alpha A p (A p = t is not stored)
+        Cx<R> pv[CPC];
+        CIO::load(a.cg_p, Vh, ch, i, pv);
+        CIO::load(a.cg_x, Vh, ch, i, v);
+#pragma unroll
+        for (int j = 0; j < CPC; ++j) {
+          v[j].re = fma(alpha, pv[j].re, v[j].re);
+          v[j].im = fma(alpha, pv[j].im, v[j].im);
+        }
+        CIO::store(a.cg_x, Vh, ch, i, v);
+        CIO::load(a.cg_r, Vh, ch, i, v);
+#pragma unroll
+        for (int j = 0; j < CPC; ++j) {
+          v[j].re = fma(-alpha, t[j].re, v[j].re);
+          v[j].im = fma(-alpha, t[j].im, v[j].im);
+          n2 += norm2(v[j]);
+        }
+        CIO::store(a.cg_r, Vh, ch, i, v);
+      } else {
+        CIO::store(a.out, Vh, ch, i, t);
+#pragma unroll
+        for (int j = 0; j < CPC; ++j) n2 += norm2(t[j]);
+      }
+    }
+  }
+  if (a.partials) {
+    // |out|^2 of a site in the arithmetic precision, across sites in double
+    // (by one warp: FP64 additions are scarce on this GPU)
+    s_n[mu][lane] = n2;
+    __syncthreads();
+    if (mu == 0) {
+      double s = (double)((s_n[0][lane] + s_n[1][lane]) + (s_n[2][lane] + s_n[3][lane]));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+      if (lane == 0) a.partials[blockIdx.x] = s;
+    }
+    if (a.total) last_block_total<SPLIT_NT>(a.partials, a.counter, a.total);
+  }
+}
+
+template <int SP, int FMT>
+void launch_fmt(const DslashArgs &a, int dagger, cudaStream_t st) {
+  const int nb = blocks_for(a.g.Vh, SPLIT_SITES);
+  if (dagger)
+    launch_pdl(k_dslash_split<SP, FMT, true>, nb, SPLIT_NT, st, a.pdl != 0, a);
+  else
+    launch_pdl(k_dslash_split<SP, FMT, false>, nb, SPLIT_NT, st, a.pdl != 0, a);
+}
+
+}  // namespace
+
+int dslash_split_blocks(const Geo &g) { return blocks_for(g.Vh, SPLIT_SITES); }
+
+// The sites of the fullest SM decide: 32-site blocks spread the lattice
+// finer than 128-site blocks, at a cost per site (coordinates four times, the
+// exchange).  Measured, one thread per site against this kernel:
+//   FP32, per CG iteration: Vh 20736 36.8 / 30.8 us, 36864 40.4 / 39.2, 65536
+//     52.8 / 53.0, 81920 56.6 / 66.0: up to 256 sites per SM.
+//   emulated FP64, per hop: 36864 32.2 / 27.7 us, 65536 54.2 / 49.3, 81920
+//     60.8 / 59.3, 128000 87.7 / 90.0: up to 2^16 sites.
+//   FP64 (bound by its pipe, 25 % dearer per site here), per CG iteration:
+//     20736 282 / 208 us, 36864 285 / 319, 65536 550 / 549, 128000 953 / 1034:
+//     where the fullest SM gets enough fewer sites.
+// The fused CG update needs alpha formed by the launch before; per-right-
+// hand-side factors belong to several right-hand sides.
+bool dslash_split_rule(const hmc_ctx *ctx, const DslashArgs &a, int sprec) {
+  if (a.n_rhs != 1 || a.cb_rhs || (a.cg_x && !a.cg_alpha)) return false;
+  const long long Vh = a.g.Vh, sms = ctx->sm_count;
+  switch (sprec) {
+    case HMC_F32: return Vh <= 256 * sms;
+    case HMC_F64E: return Vh <= 1 << 16;
+    case HMC_F64: {
+      const long long fine = (Vh + SPLIT_SITES * sms - 1) / (SPLIT_SITES * sms) * SPLIT_SITES;
+      const long long coarse = (Vh + DS_NT * sms - 1) / (DS_NT * sms) * DS_NT;
+      return 5 * fine < 4 * coarse;
+    }
+    default: return false;
+  }
+}
+
+bool launch_dslash_split(const DslashArgs &a, int sprec, int fmt, int dagger, cudaStream_t st) {
+  switch (sprec * 100 + fmt) {
+    case HMC_F64 * 100 + 18: launch_fmt<HMC_F64, 18>(a, dagger, st); return true;
+    case HMC_F64 * 100 + 12: launch_fmt<HMC_F64, 12>(a, dagger, st); return true;
+    case HMC_F32 * 100 + 18: launch_fmt<HMC_F32, 18>(a, dagger, st); return true;
+    case HMC_F32 * 100 + 12: launch_fmt<HMC_F32, 12>(a, dagger, st); return true;
+    case HMC_F64E * 100 + 18: launch_fmt<HMC_F64E, 18>(a, dagger, st); return true;
+    case HMC_F64E * 100 + 12: launch_fmt<HMC_F64E, 12>(a, dagger, st); return true;
+    default: return false;
+  }
+}
+
+}  // namespace hmc

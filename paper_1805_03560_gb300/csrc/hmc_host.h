@@ -204,7 +204,17 @@ struct DslashArgs {
   // > 0: launch the multi-right-hand-side kernel with this many right-hand
   // sides per thread (set by callers that need its fused epilogue)
   int mr_force;
+  // nothing still running on the stream writes the links (set inside a
+  // solve): the one-thread-per-direction kernel may load them before its wait for
+  // the launch before
+  int links_ready;
 };
+// One-thread-per-direction hemi-Dslash (dslash_split.cu) of one right-hand
+// side: whether it is the kernel for this launch, its launch, and its block
+// count (the partials it leaves; the kernels of DS_NT threads leave fewer).
+bool dslash_split_rule(const hmc_ctx *ctx, const DslashArgs &a, int sprec);
+bool launch_dslash_split(const DslashArgs &a, int sprec, int fmt, int dagger, cudaStream_t st);
+int dslash_split_blocks(const Geo &g);
 // Multi-right-hand-side hemi-Dslash with nr right-hand sides per thread
 // (dslash_mr.cu): FP32 or FP16 storage, 2 <= nr <= 4 dividing n_rhs <= 16.
 bool dslash_mr_supported(int sprec, int n_rhs, int nr);

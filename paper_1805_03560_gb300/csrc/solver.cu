@@ -518,6 +518,7 @@ int one_iteration(Solve &s, int k) {
   a.gauge = U.data;
   a.gate = &s.st->active;
   a.tag = "cg";
+  a.links_ready = 1;
   // t = H_oe p; y = p - kappa^2 H_eo t with |y|^2 block partials
   a.p = 1; a.out = s.tlo; a.in = s.p; a.cb = 1.0;
   TRY(dslash(ctx, a, U, s.plo, 0, nullptr));
@@ -802,7 +803,7 @@ int cg_solve(hmc_ctx *ctx, const Geo &g, const hmc_gauge &Uh, const hmc_gauge *U
   s.kappa = kappa;
   TRY(hi_begin(ctx, g, Uh, opts, &s.hi, "cg"));
   s.S = g.Vh;
-  s.nb_ds = blocks_for(g.Vh, DS_NT);
+  s.nb_ds = dslash_split_blocks(g);
   s.nb_bl = blocks_for(g.Vh, BL_NT);
   const size_t f64 = spinor_bytes(g, HMC_F64, 1);
   const size_t f32 = spinor_bytes(g, HMC_F32, 1);
