@@ -244,7 +244,7 @@ template <int SP, int FMT>
 __device__ __forceinline__ void prefetch_block_links(const DslashArgs &a) {
   const int t = threadIdx.x;
   if (t >= 8) return;
-  const int Vh = a.g.Vh, h0 = blockIdx.x * DS_NT, mu = t >> 1;
+  const int Vh = a.g.Vh, h0 = ds_block(a) * DS_NT, mu = t >> 1;
   const bool fwd = (t & 1) == 0;
   const int sh = fwd ? 0 : (mu == 3 ? 1 : a.g.st[mu] >> 1);
   int lo = h0 - sh, hi = h0 + DS_NT - sh + (!fwd && mu == 3 ? 1 : 0);
@@ -308,9 +308,9 @@ __device__ __forceinline__ void hops_rt(const DslashArgs &a, int h, int r, int l
 // 32 consecutive sites each at the offsets {0, +x, +t, +x+t}, so half of the
 // x and t neighbours a block reads are its own sites and can hit in L1.
 __device__ __forceinline__ int dslash_site(const DslashArgs &a) {
-  if (a.tile_nseg == 0) return blockIdx.x * DS_NT + threadIdx.x;
+  if (a.tile_nseg == 0) return ds_block(a) * DS_NT + threadIdx.x;
   const int sx = a.g.L[2] * a.g.Lzh, st = a.g.L[1] * sx;
-  const int b = blockIdx.x;
+  const int b = ds_block(a);
   const int seg = b % a.tile_nseg, xt = b / a.tile_nseg;
   const int hx = a.g.L[1] >> 1;
   const int xp = xt % hx, tp = xt / hx;
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(DS_NT, ds_min_blocks(SP)) k_dslash(const Dslas
   if (a.partials) {
     if (a.n_rhs == 1) {
       double s = block_sum<DS_NT>(nrm);
-      if (threadIdx.x == 0) a.partials[blockIdx.x] = s;
+      if (threadIdx.x == 0) a.partials[ds_block(a)] = s;
       if (a.total) last_block_total<DS_NT>(a.partials, a.counter, a.total);
     } else {
       // one partial (and total) per right-hand side
@@ -691,6 +691,9 @@ int dslash(hmc_ctx *ctx, const DslashArgs &a, const hmc_gauge &U, int sprec, int
     *nblocks = blocks_for((long long)a.g.Vh * (a.n_rhs / (var - 2)), DS_NT);
   DslashArgs la = a;
   la.pdl = ctx->pdl;
+  // every launch walks the lattice the other way (ds_block); block totals and
+  // per-right-hand-side partials are stored in launch order and stay so
+  if (!a.total && !(a.partials && a.n_rhs > 1)) la.rev = ctx->ds_rev ^= 1;
   if (split) {
     if (nblocks) *nblocks = dslash_split_blocks(a.g);
     TimedLaunch timer(ctx, cls, bytes);

@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(DS_NT, mr_min_blocks(NR)) k_dslash_mr(const Ds
   griddep_wait();
   if (a.gate && *a.gate == 0) return;
   const int n = a.n_rhs, NG = n / NR, St = a.g.Vh * n;
-  const int i = blockIdx.x * DS_NT + threadIdx.x;
+  const int i = ds_block(a) * DS_NT + threadIdx.x;
   double nrm[NR];
   int rr[NR];
 #pragma unroll

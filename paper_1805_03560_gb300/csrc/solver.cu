@@ -159,16 +159,22 @@ __global__ void __launch_bounds__(BL_NT) k_dot(const void *x, const void *y, int
 template <int PL>
 __global__ void __launch_bounds__(BL_NT) k_cg_xpay(void *p, const void *r, int S, CGState *st,
                                                    int par, int plain, const double *rr_part,
-                                                   int n_part) {
+                                                   int n_part, int rev) {
   griddep_launch_dependents();
   griddep_wait();
   if (!st->active) return;
   using R = RT<PL>;
   // the first grid-stride element's r and p are loaded before the sum of the
   // partials, so that their DRAM latency overlaps the reduction
-  const int i0 = blockIdx.x * BL_NT + threadIdx.x;
+  const int j0 = blockIdx.x * BL_NT + threadIdx.x;
+  // rev: from the last element to the first (the launch before, the fused
+  // update, went the other way and left its last elements in L2); top makes
+  // groups of 32 consecutive threads whole groups of 32 elements
+  const int top = ((S + 31) & ~31) - 1;
+  const auto at = [&](int j) { return rev ? top - j : j; };
+  const int i0 = at(j0);
   Cx<R> rv[12], pv[12];
-  if (i0 < S) {
+  if (j0 <= top && i0 < S) {
     load_as<PL>(r, S, i0, rv);
     load_as<PL>(p, S, i0, pv);
   }
@@ -199,19 +205,21 @@ __global__ void __launch_bounds__(BL_NT) k_cg_xpay(void *p, const void *r, int S
   // partials; the next element's loads are issued before the current one is
   // updated, two elements in flight per thread
   const int stride = gridDim.x * BL_NT;
-  for (int i = i0; i < S; i += stride) {
+  for (int j = j0; j <= top; j += stride) {
     Cx<R> rn[12], pn[12];
-    const int in = i + stride;
-    if (in < S) {
+    const int i = at(j), in = at(j + stride);
+    if (j + stride <= top && in < S) {
       load_as<PL>(r, S, in, rn);
       load_as<PL>(p, S, in, pn);
     }
+    if (i < S) {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      pv[k].re = fma(beta, pv[k].re, rv[k].re);
-      pv[k].im = fma(beta, pv[k].im, rv[k].im);
+      for (int k = 0; k < 12; ++k) {
+        pv[k].re = fma(beta, pv[k].re, rv[k].re);
+        pv[k].im = fma(beta, pv[k].im, rv[k].im);
+      }
+      store_as<PL>(p, S, i, pv);
     }
-    store_as<PL>(p, S, i, pv);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
       rv[k] = rn[k];
@@ -497,7 +505,8 @@ template <int PL>
 void launch_xpay(Solve &s, int par, int n_part) {
   const int nb = s.nb_bl < 2 * s.ctx->sm_count ? s.nb_bl : 2 * s.ctx->sm_count;
   launch_pdl(k_cg_xpay<PL>, nb, BL_NT, s.ctx->stream, s.ctx->pdl != 0, s.p, (const void *)s.rlo,
-             s.S, s.st, par, s.plo == HMC_F64 ? 1 : 0, (const double *)s.rr_part, n_part);
+             s.S, s.st, par, s.plo == HMC_F64 ? 1 : 0, (const double *)s.rr_part, n_part,
+             s.ctx->ds_rev ^= 1);
 }
 
 // One iteration, five launches: y = Mhat p (the second hemi-Dslash leaves
