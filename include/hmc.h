@@ -165,8 +165,8 @@ int hmc_ctx_set_timing(hmc_ctx *ctx, int enable);
  * read (12-real FP32, F16 and BF16 links, one right-hand side; bit-identical
  * results; elsewhere variant 0 or 2 runs).  Default -1: for n_rhs > 1 in
  * FP32/FP16 the multi-right-hand-side kernel with 2 (else 3) per thread where
- * that divides n_rhs, otherwise paired loads for LINK18 only (the fastest
- * choice measured on 24^3 x 48).  With -1 and -2, one right-hand side in FP64,
+ * that divides n_rhs, otherwise paired loads for LINK18, for half storage and,
+ * in FP32, where they fill the GPU better (by the lattice size).  With -1 and -2, one right-hand side in FP64,
  * FP32 or emulated FP64 on a lattice too small to fill the GPU runs one thread
  * per site and direction (the four directions' sums added last: within
  * rounding of the other variants).  -2: autotune: the first launch of each class

@@ -323,10 +323,17 @@ __device__ __forceinline__ int dslash_site(const DslashArgs &a) {
 // register count allows, so fewer registers (more warps in flight) win as
 // long as nothing spills.  Measured on 24^3x48: FP32 storage at 6 blocks
 // (80 registers, no spills) 39.1 us against 41.4 us at 5 blocks (100
-// registers); the FP64 kinds gain nothing.  Half storage (F16, BF16) at 4
+// registers); the FP64 kinds gain nothing.  The paired FP32 form at 4 blocks
+// (128 registers): loads in flight instead of threads, for lattices that do not
+// fill six blocks per SM (default_variant); 18-real links gain at every size
+// (CG iteration 16^3x32 58.1 -> 45.9 us, 24^3x48 231 -> 224 us, 32^3x64 703 -> 654
+// us against 6 blocks).  Half storage (F16, BF16) at 4
 // blocks: its four-hop load form then fits in 128 registers without spills.
 #ifndef HMC_DS_MINB32
 #define HMC_DS_MINB32 6
+#endif
+#ifndef HMC_DS_MINB32P
+#define HMC_DS_MINB32P 4
 #endif
 #ifndef HMC_DS_MINB16
 #define HMC_DS_MINB16 4
@@ -340,8 +347,8 @@ __device__ __forceinline__ int dslash_site(const DslashArgs &a) {
 #ifndef HMC_DS_MINBBF16
 #define HMC_DS_MINBBF16 4
 #endif
-constexpr int ds_min_blocks(int sp) {
-  return sp == HMC_F32    ? HMC_DS_MINB32
+constexpr int ds_min_blocks(int sp, int fmt, bool pair) {
+  return sp == HMC_F32    ? (pair ? HMC_DS_MINB32P : HMC_DS_MINB32)
          : sp == HMC_F16  ? HMC_DS_MINB16
          : sp == HMC_BF16 ? HMC_DS_MINBBF16
          : sp == HMC_F64E ? HMC_DS_MINB64E
@@ -349,7 +356,7 @@ constexpr int ds_min_blocks(int sp) {
 }
 
 template <int SP, int FMT, bool DAG, bool PAIR>
-__global__ void __launch_bounds__(DS_NT, ds_min_blocks(SP)) k_dslash(const DslashArgs a) {
+__global__ void __launch_bounds__(DS_NT, ds_min_blocks(SP, FMT, PAIR)) k_dslash(const DslashArgs a) {
   using SIO = SpinorIO<SP>;
   using R = typename SIO::R;
   constexpr int SF = DAG ? -1 : 1;  // forwards: 1 - gamma (1 + gamma for the adjoint)
@@ -546,10 +553,27 @@ static int mr_default(int sprec, int n_rhs) {
   return 0;
 }
 
-static int default_variant(int fmt, int sprec, int n_rhs) {
+// Built-in variant of a launch of nb blocks (sites x right-hand sides over
+// DS_NT).  18-real links: paired loads.  Half storage with 12-real links, one
+// right-hand side: the four-hop loads (a CG iteration in F16 45.9 us against
+// 47.7 on 16^3 x 32, 157.0 against 166.5 on 24^3 x 48, 456.7 against 485.1 on
+// 32^3 x 64).  FP32 with 12-real links: paired loads in 128 registers (four
+// blocks per SM) keep more loads in flight per thread, the single form in 80
+// (six per SM) more threads; per SM filled they are within 2 % of each other,
+// so the one whose last wave is fuller wins (CG iteration, single / paired:
+// 16^3 x 32, 512 blocks, 52.0 / 43.6 us; 16^3 x 40 56.5 / 57.2; 20^3 x 32 89.5 /
+// 79.7; 20^3 x 48 115.7 / 118.4; 24^3 x 48 187.3 / 193.9), and from eight waves
+// on, where the last one counts little, the paired form (32^3 x 64 564.0 /
+// 557.7).
+static int default_variant(const hmc_ctx *ctx, int fmt, int sprec, int n_rhs, int nb) {
   const int nr = mr_default(sprec, n_rhs);
   if (nr) return 2 + nr;
-  return fmt == 18 ? 2 : 0;
+  if (fmt == 18) return 2;
+  if (n_rhs > 1) return 0;
+  if (sprec == HMC_F16 || sprec == HMC_BF16) return 2;
+  if (sprec != HMC_F32) return 0;
+  const int w4 = blocks_for(nb, 4 * ctx->sm_count), w6 = blocks_for(nb, 6 * ctx->sm_count);
+  return w4 == 1 || w4 >= 8 || 4 * w4 < 6 * w6 ? 2 : 0;
 }
 
 // whether variants 7 and 8 (links prefetched into L2) apply
@@ -587,7 +611,7 @@ static int tune_variant(hmc_ctx *ctx, const DslashArgs &a, int sprec, int fmt, i
                           a.out != a.x && a.out != a.in;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(ctx->stream, &cs);
-  const int dflt = default_variant(fmt, sprec, a.n_rhs);
+  const int dflt = default_variant(ctx, fmt, sprec, a.n_rhs, nb);
   if (!repeatable || cs != cudaStreamCaptureStatusNone || ctx->tune_frozen) return dflt;
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess) return dflt;
@@ -668,10 +692,9 @@ int dslash(hmc_ctx *ctx, const DslashArgs &a, const hmc_gauge &U, int sprec, int
            U.fmt, a.tag ? "/" : "",
            a.tag ? a.tag : "");
   // kernel variant (hmc_ctx_set_option): bit 0 tiled site mapping, bit 1
-  // paired loads.  Default -1: paired loads for 18-real links only (measured
-  // on 24^3 x 48, pairing helps the 18-real kernels and slows the 12-real
-  // ones, tiling helps neither); -2: autotuned per class.
-  int var = ctx->ds_variant >= 0 ? ctx->ds_variant : default_variant(U.fmt, sprec, a.n_rhs);
+  // paired loads.  Default -1: default_variant (tiling measured slower);
+  // -2: autotuned per class.
+  int var = ctx->ds_variant >= 0 ? ctx->ds_variant : default_variant(ctx, U.fmt, sprec, a.n_rhs, nb);
   // small lattices: one thread per direction, unless a variant is asked for
   const bool split = ctx->ds_variant < 0 && dslash_split_rule(ctx, a, sprec);
   if (ctx->ds_variant == -2 && !split) var = tune_variant(ctx, a, sprec, U.fmt, dagger, nb);
