@@ -270,7 +270,9 @@ int kinetic_partials(hmc_ctx *ctx, const Geo &g, const double *P, double *partia
 // emulated FP64 (the projection stays FP64)
 int update_links(hmc_ctx *ctx, const Geo &g, void *U, const double *P, double eps,
                  bool emul = false);
-int convert_gauge(hmc_ctx *ctx, const Geo &g, const void *src, void *dst, int prec, int fmt);
+// src: F64 links in format src_fmt
+int convert_gauge(hmc_ctx *ctx, const Geo &g, const void *src, void *dst, int prec, int fmt,
+                  int src_fmt = HMC_LINK18);
 int cg_solve(hmc_ctx *ctx, const Geo &g, const hmc_gauge &Uh, const hmc_gauge *Ul, void *x,
              const void *b, double kappa, double tol, int max_iter, const hmc_solver_opts *opts,
              hmc_solve_stats *stats);

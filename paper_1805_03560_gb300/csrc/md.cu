@@ -317,14 +317,14 @@ __global__ void __launch_bounds__(128) k_update_links_e(Geo g, void *gauge, cons
   LinkIO<HMC_F64, 18>::store(base, g.Vh, h, u);
 }
 
-// F64/LINK18 -> any precision / format (same site order)
-template <int P, int FMT>
+// F64 links (LINK18 unless SFMT says otherwise) -> any precision / format (same site order)
+template <int P, int FMT, int SFMT = 18>
 __global__ void k_convert_gauge(Geo g, const void *src, void *dst) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 8 * g.Vh) return;
   const int pm = i / g.Vh, h = i - pm * g.Vh;
   C u[9];
-  LinkIO<HMC_F64, 18>::load((const char *)src + (size_t)pm * 9 * g.Vh * 16, g.Vh, h, u);
+  LinkIO<HMC_F64, SFMT>::load(link_base<HMC_F64, SFMT>(src, g.Vh, pm >> 2, pm & 3), g.Vh, h, u);
   LinkIO<P, FMT>::store((void *)link_base<P, FMT>(dst, g.Vh, pm >> 2, pm & 3), g.Vh, h, u);
 }
 
@@ -350,9 +350,16 @@ int update_links(hmc_ctx *ctx, const Geo &g, void *U, const double *P, double ep
   return launched(ctx, "update_links");
 }
 
-int convert_gauge(hmc_ctx *ctx, const Geo &g, const void *src, void *dst, int prec, int fmt) {
+int convert_gauge(hmc_ctx *ctx, const Geo &g, const void *src, void *dst, int prec, int fmt,
+                  int src_fmt) {
   int nb = blocks_for(8LL * g.Vh, 256);
   cudaStream_t st = ctx->stream;
+  if (src_fmt == 12) {
+    if (prec != HMC_F64E || fmt != 12)
+      return fail(ctx, HMC_EINVAL, "convert_gauge: 12-real links convert to F64E/LINK12 only");
+    k_convert_gauge<HMC_F64E, 12, 12><<<nb, 256, 0, st>>>(g, src, dst);
+    return launched(ctx, "convert_gauge");
+  }
   switch (prec * 100 + fmt) {
     case HMC_F64 * 100 + 18: k_convert_gauge<HMC_F64, 18><<<nb, 256, 0, st>>>(g, src, dst); break;
     case HMC_F64 * 100 + 12: k_convert_gauge<HMC_F64, 12><<<nb, 256, 0, st>>>(g, src, dst); break;

@@ -152,7 +152,7 @@ int force_links(hmc_ctx *ctx, const Geo &g, const hmc_gauge &Uh, const hmc_gauge
   if (fp == HMC_F64E) {
     void *ue = workspace(ctx, "pf_ue", gauge_bytes(g, HMC_F64E, Uh.fmt));
     if (!ue) return HMC_ENOMEM;
-    TRY(convert_gauge(ctx, g, Uh.data, ue, HMC_F64E, Uh.fmt));
+    TRY(convert_gauge(ctx, g, Uh.data, ue, HMC_F64E, Uh.fmt, Uh.fmt));
     *Uf = hmc_gauge{ue, HMC_F64E, Uh.fmt};
     return HMC_OK;
   }
