@@ -517,7 +517,7 @@ static bool launch_variant(const DslashArgs &a, int sprec, int fmt, int dagger, 
     case HMC_F16 * 100 + 12: launch_sf<HMC_F16, 12>(aa, dagger, pair, nb, st); break;
     case HMC_BF16 * 100 + 18: launch_sf<HMC_BF16, 18>(aa, dagger, pair, nb, st); break;
     case HMC_BF16 * 100 + 12: launch_sf<HMC_BF16, 12>(aa, dagger, pair, nb, st); break;
-    case HMC_F64E * 100 + 18: launch_sf<HMC_F64E, 18>(aa, dagger, pair, nb, st); break;
+    case HMC_F64E * 100 + 18: launch_dslash_e2(aa, dagger, st); break;
     case HMC_F64E * 100 + 12: launch_sf<HMC_F64E, 12>(aa, dagger, pair, nb, st); break;
     default: return false;
   }

@@ -18,7 +18,7 @@
 // kernel): a CG iteration in FP32 on 8^3 x 16 33.1 -> 23.2 us, on 14 x 6 x 10
 // x 20 33.7 -> 24.8 us, on 12^3 x 24 36.8 -> 30.8 us; in FP64 155 -> 84, 201 ->
 // 131 and 282 -> 208 us; the emulated-FP64 hop 22.0 -> 9.7, 22.8 -> 10.8 and 30.4
-// -> 18.2 us.  (One thread per hop, eight warps to 32 sites, was slower for
+// -> 18.2 us (16.1 in the paired arithmetic).  (One thread per hop, eight warps to 32 sites, was slower for
 // FP32: 38.6 us per iteration on 12^3 x 24, the barrier's traffic doubles.)
 #include "dslash_ops.cuh"
 #include "hmc_host.h"
@@ -72,26 +72,6 @@ struct ChunkIO<HMC_F64E> {
   }
 };
 
-// project and accumulate of a direction known at run time (uniform over a warp)
-template <int S, typename R>
-__device__ __forceinline__ void project_mu(int mu, const Cx<R> p[12], Cx<R> h[6]) {
-  switch (mu) {
-    case 0: project<0, S>(p, h); break;
-    case 1: project<1, S>(p, h); break;
-    case 2: project<2, S>(p, h); break;
-    default: project<3, S>(p, h); break;
-  }
-}
-template <int S, typename R>
-__device__ __forceinline__ void accumulate_mu(int mu, Cx<R> acc[12], const Cx<R> w[6]) {
-  switch (mu) {
-    case 0: accumulate<0, S>(acc, w); break;
-    case 1: accumulate<1, S>(acc, w); break;
-    case 2: accumulate<2, S>(acc, w); break;
-    default: accumulate<3, S>(acc, w); break;
-  }
-}
-
 // fermion boundary sign of a hop in time that wraps around
 template <typename R>
 __device__ __forceinline__ void flip(bool wrap, Cx<R> h[6]) {
@@ -138,20 +118,34 @@ __global__ void __launch_bounds__(SPLIT_NT, split_min_blocks<SP>()) k_dslash_spl
   if constexpr (SP == HMC_F64E) {
     griddep_wait();
     if (a.gate && *a.gate == 0) return;
+    AccE2 e2;
+    if constexpr (FMT == 18) zero_e2(e2);
 #pragma unroll 1
     for (int d = 0; d < 2; ++d) {
-      Cx<R> psi[12], u[9], hs[6], w[6];
-      SIO::load(a.in, Vh, d ? hb : hf, psi);
-      LIO::load(d ? gb : gf, Vh, d ? hb : is, u);
       const int S = d ? -SF : SF;
-      project_rt(mu, S, psi, hs);
-      flip(d ? wb : wf, hs);
-      if (d)
-        mul_link_dag(u, hs, w);
-      else
-        mul_link(u, hs, w);
-      accumulate_rt(mu, S, acc, w);
+      if constexpr (FMT == 18) {
+        const float4 *in = (const float4 *)a.in + (d ? hb : hf);
+        const float4 *lk = (const float4 *)(d ? gb : gf) + (d ? hb : is);
+        float4 p[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) p[k] = __ldg(in + (size_t)k * Vh);
+        const size_t sr = (size_t)(d ? 1 : 3) * Vh, sc = (size_t)(d ? 3 : 1) * Vh;
+        hop_e2(p, [] {}, [&](int r, int k) { return __ldg(lk + r * sr + k * sc); }, mu, d == 0,
+               S, d ? wb : wf, e2);
+      } else {
+        Cx<R> psi[12], u[9], hs[6], w[6];
+        SIO::load(a.in, Vh, d ? hb : hf, psi);
+        LIO::load(d ? gb : gf, Vh, d ? hb : is, u);
+        project_rt(mu, S, psi, hs);
+        flip(d ? wb : wf, hs);
+        if (d)
+          mul_link_dag(u, hs, w);
+        else
+          mul_link(u, hs, w);
+        accumulate_rt(mu, S, acc, w);
+      }
     }
+    if constexpr (FMT == 18) unpack_e2(e2, acc);
   } else {
     Cx<R> uf[9], ub[9], pf[12], pb[12], hs[6], w[6];
     if (!a.links_ready) griddep_wait();
@@ -267,8 +261,8 @@ int dslash_split_blocks(const Geo &g) { return blocks_for(g.Vh, SPLIT_SITES); }
 // exchange).  Measured, one thread per site against this kernel:
 //   FP32, per CG iteration: Vh 20736 36.8 / 30.8 us, 36864 40.4 / 39.2, 65536
 //     52.8 / 53.0, 81920 56.6 / 66.0: up to 256 sites per SM.
-//   emulated FP64, per hop: 36864 32.2 / 27.7 us, 65536 54.2 / 49.3, 81920
-//     60.8 / 59.3, 128000 87.7 / 90.0: up to 2^16 sites.
+//   emulated FP64, per hop: 20736 33.0 / 16.1 us, 36864 33.3 / 24.4, 65536
+//     41.6 / 45.7, 81920 50.2 / 50.3: up to 384 sites per SM.
 //   FP64 (bound by its pipe, 25 % dearer per site here), per CG iteration:
 //     20736 282 / 208 us, 36864 285 / 319, 65536 550 / 549, 128000 953 / 1034:
 //     where the fullest SM gets enough fewer sites.
@@ -279,7 +273,7 @@ bool dslash_split_rule(const hmc_ctx *ctx, const DslashArgs &a, int sprec) {
   const long long Vh = a.g.Vh, sms = ctx->sm_count;
   switch (sprec) {
     case HMC_F32: return Vh <= 256 * sms;
-    case HMC_F64E: return Vh <= 1 << 16;
+    case HMC_F64E: return Vh <= 384 * sms;
     case HMC_F64: {
       const long long fine = (Vh + SPLIT_SITES * sms - 1) / (SPLIT_SITES * sms) * SPLIT_SITES;
       const long long coarse = (Vh + DS_NT * sms - 1) / (DS_NT * sms) * DS_NT;

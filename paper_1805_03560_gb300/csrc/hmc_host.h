@@ -223,6 +223,9 @@ struct DslashArgs {
 __device__ __forceinline__ int ds_block(const DslashArgs &a) {
   return a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
 }
+// Emulated FP64 with 18-real links, one thread per site and right-hand side
+// (dslash_e2.cu)
+void launch_dslash_e2(const DslashArgs &a, int dagger, cudaStream_t st);
 // One-thread-per-direction hemi-Dslash (dslash_split.cu) of one right-hand
 // side: whether it is the kernel for this launch, its launch, and its block
 // count (the partials it leaves; the kernels of DS_NT threads leave fewer).
@@ -279,20 +282,17 @@ int cg_solve(hmc_ctx *ctx, const Geo &g, const hmc_gauge &Uh, const hmc_gauge *U
 
 // BiCGstab on Mhat (dagger 0) or Mhat^dag, and (Mhat^dag Mhat)^{-1} as two
 // such solves (bicgstab.cu)
-// kernel<<<nb, nt, 0, st>>>(args...), as a programmatic dependent launch
-// (cudaLaunchAttributeProgrammaticStreamSerialization) when pdl: the kernel
-// must then call griddep_wait() before touching the previous kernel's data
 template <typename... KArgs, typename... Args>
-inline void launch_pdl(void (*kernel)(KArgs...), int nb, int nt, cudaStream_t st, bool pdl,
-                       Args... args) {
+inline void launch_pdl_smem(void (*kernel)(KArgs...), int nb, int nt, size_t smem, cudaStream_t st,
+                            bool pdl, Args... args) {
   if (!pdl) {
-    kernel<<<nb, nt, 0, st>>>(args...);
+    kernel<<<nb, nt, smem, st>>>(args...);
     return;
   }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(nb);
   cfg.blockDim = dim3(nt);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -300,6 +300,15 @@ inline void launch_pdl(void (*kernel)(KArgs...), int nb, int nt, cudaStream_t st
   cfg.attrs = at;
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// kernel<<<nb, nt, 0, st>>>(args...), as a programmatic dependent launch
+// (cudaLaunchAttributeProgrammaticStreamSerialization) when pdl: the kernel
+// must then call griddep_wait() before touching the previous kernel's data
+template <typename... KArgs, typename... Args>
+inline void launch_pdl(void (*kernel)(KArgs...), int nb, int nt, cudaStream_t st, bool pdl,
+                       Args... args) {
+  launch_pdl_smem(kernel, nb, nt, 0, st, pdl, args...);
 }
 
 // the context's graph-replay stream, its two ordering events and the two
