@@ -14,6 +14,7 @@
 // staple sum A of U_{x,mu}, S_G = -(beta/3) Re Tr(U A) + ..., so
 // F_a = (beta/6) Im Tr(lambda_a U A); a Polyakov line through the link
 // contributes -64 kappa^4 s_mu Im Tr(lambda_a P_mu(x)) (the line starting at x).
+#include "df64x2.cuh"
 #include "hmc_host.h"
 
 namespace hmc {
@@ -104,6 +105,35 @@ struct GaugeArgs {
   double *partials; // action kernel: [block] plaquette sums, [nblocks + block] line sums
 };
 
+// F += cplaq Im Tr(lambda (U A)) (and the line through the link); u1: the link, t = U A
+template <int P, int FMT>
+__device__ __forceinline__ void add_gauge_force(const GaugeArgs &a, const int c[4], int p, int mu,
+                                                int h, const Cx<typename LinkIO<P, FMT>::R> u1[9],
+                                                Cx<typename LinkIO<P, FMT>::R> t[9]) {
+  using C = Cx<typename LinkIO<P, FMT>::R>;
+  C u2[9], u3[9];
+  double f[8], fp[8];
+  im_tr_lambda_g(t, f);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) f[k] *= a.cplaq;
+  const double cp = a.cpoly[mu];
+  if (cp != 0.0) {
+    // P = U_{x,mu} U_{x+mu,mu} ... around the torus (extent 4)
+    for (int k = 0; k < 9; ++k) t[k] = u1[k];
+    for (int s = 1; s < a.g.L[mu]; ++s) {
+      link_at<P, FMT>(a.g, a.gauge, c, mu, mu, s, 0, 0, u2);
+      m_mul(t, u2, u3);
+      for (int k = 0; k < 9; ++k) t[k] = u3[k];
+    }
+    im_tr_lambda_g(t, fp);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) f[k] += cp * fp[k];
+  }
+  double *F = a.F + (size_t)(p * 4 + mu) * 8 * a.g.Vh + h;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) F[(size_t)k * a.g.Vh] += f[k];
+}
+
 template <int P, int FMT>
 __global__ void __launch_bounds__(128) k_gauge_force(const GaugeArgs a) {
   using R = typename LinkIO<P, FMT>::R;
@@ -140,26 +170,116 @@ __global__ void __launch_bounds__(128) k_gauge_force(const GaugeArgs a) {
   }
   link_at<P, FMT>(a.g, a.gauge, c, mu, 0, 0, 0, 0, u1);
   m_mul(u1, A, t);
-  double f[8], fp[8];
-  im_tr_lambda_g(t, f);
+  add_gauge_force<P, FMT>(a, c, p, mu, h, u1, t);
+}
+
+// Emulated FP64 with 18-real links: the upper and the lower staple of a plane
+// in the two lanes of the paired arithmetic (df64x2.cuh).  Both are products
+// X Y Z of three links or adjoints (an adjoint: indices exchanged by the load,
+// imaginary parts negated):
+//   upper  U_{x+mu,nu}            U^dag_{x+nu,mu}   U^dag_{x,nu}
+//   lower  U^dag_{x+mu-nu,nu}     U^dag_{x-nu,mu}   U_{x-nu,nu}
+// A staple is built as sum_k X[:,k] (Y[k,:] Z): Z sits in shared memory, one
+// row of Y and one column of X are read per step and the staple stays in
+// registers, so the loop over planes and k holds two sets of nine complex
+// products (the scalar kernel, unrolled, is several times the instruction
+// cache: 2.0 of its 3.6 stall cycles per issue were waits for instructions).
+// The sum A over the planes is kept in shared memory: adding every plane's
+// products into one accumulator instead would round each of them at the size
+// of the sum (measured: 3.4e-15 off the exact force, against 3.1e-15).
+constexpr int GF_NT = 128;
+constexpr int GF_SMEM = 2 * 9 * 2 * GF_NT * 16;
+
+__device__ __forceinline__ cdd2 pair_elements(float4 up, float4 lo, f32x2 im_mask) {
+  return {{pk2(up.x, lo.x), pk2(up.y, lo.y)},
+          {pk2(up.z, lo.z) ^ im_mask, pk2(up.w, lo.w) ^ im_mask}};
+}
+
+__global__ void __launch_bounds__(GF_NT, 3) k_gauge_force_e2(const GaugeArgs a) {
+  extern __shared__ __align__(16) ulonglong2 s_z[];  // Z and A: [9][re, im][thread] each
+  const int nb_pm = (a.g.Vh + GF_NT - 1) / GF_NT;
+  const int pm = blockIdx.x / nb_pm, p = pm & 1, mu = pm >> 1;
+  const int h = (blockIdx.x - pm * nb_pm) * GF_NT + threadIdx.x;
+  if (h >= a.g.Vh) return;
+  const int Vh = a.g.Vh;
+  int c[4];
+  const int lex = site_coords(a.g, h, p, c);
+  // displacement in lex of one step along d from coordinate x, forwards and backwards
+  const auto fw = [&](int d, int x) { return (x + 1 == a.g.L[d] ? 1 - a.g.L[d] : 1) * a.g.st[d]; };
+  const auto bw = [&](int d, int x) { return (x == 0 ? a.g.L[d] - 1 : -1) * a.g.st[d]; };
+  const auto coord = [&](int d) { return d == 0 ? c[0] : d == 1 ? c[1] : d == 2 ? c[2] : c[3]; };
+  const auto at = [&](int lx, int par, int d) {
+    return (const float4 *)link_base<HMC_F64E, 18>(a.gauge, Vh, par, d) + (lx >> 1);
+  };
+  ulonglong2 *z = s_z + threadIdx.x, *sum = z + 18 * GF_NT;
+  cdd2 A[9];
+  bool first_plane = true;
+  const int dmu = fw(mu, coord(mu));
+  const size_t v1 = Vh, v3 = 3 * v1;
+#pragma unroll 1
+  for (int nu = 0; nu < 4; ++nu) {
+    if (nu == mu) continue;
+    const int df = fw(nu, coord(nu)), db = bw(nu, coord(nu));
+    const float4 *xu = at(lex + dmu, 1 - p, nu), *xl = at(lex + dmu + db, p, nu);
+    const float4 *yu = at(lex + df, 1 - p, mu), *yl = at(lex + db, 1 - p, mu);
+    const float4 *zu = at(lex, p, nu), *zl = at(lex + db, 1 - p, nu);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) f[k] *= a.cplaq;
-  const double cp = a.cpoly[mu];
-  if (cp != 0.0) {
-    // P = U_{x,mu} U_{x+mu,mu} ... around the torus (extent 4)
-    for (int k = 0; k < 9; ++k) t[k] = u1[k];
-    for (int s = 1; s < a.g.L[mu]; ++s) {
-      link_at<P, FMT>(a.g, a.gauge, c, mu, mu, s, 0, 0, u2);
-      m_mul(t, u2, u3);
-      for (int k = 0; k < 9; ++k) t[k] = u3[k];
+    for (int e = 0; e < 9; ++e) {
+      const int et = (e % 3) * 3 + e / 3;
+      const cdd2 v = pair_elements(__ldg(zu + (size_t)et * Vh), __ldg(zl + (size_t)e * Vh), kNeg0);
+      z[(2 * e) * GF_NT] = make_ulonglong2(v.re.h, v.re.l);
+      z[(2 * e + 1) * GF_NT] = make_ulonglong2(v.im.h, v.im.l);
     }
-    im_tr_lambda_g(t, fp);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) f[k] += cp * fp[k];
+    for (int e = 0; e < 9; ++e) A[e] = {{0ull, 0ull}, {0ull, 0ull}};
+#pragma unroll 1
+    for (int k = 0; k < 3; ++k) {
+      // P = Y[k,:] Z, (Y)_{kl} = conj(U[l][k]) in both lanes
+      cdd2 P[3];
+#pragma unroll
+      for (int l = 0; l < 3; ++l) {
+        const cdd2 y = pair_elements(__ldg(yu + l * v3), __ldg(yl + l * v3), 0ull);
+        const cdd2 yc = {y.re, flip2(y.im, kNegBoth)};
+        const cneg2 ny = {flip2(y.re, kNegBoth), y.im};
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const ulonglong2 zr = z[(2 * (l * 3 + j)) * GF_NT], zi = z[(2 * (l * 3 + j) + 1) * GF_NT];
+          const cdd2 u = {{zr.x, zr.y}, {zi.x, zi.y}};
+          P[j] = l == 0 ? cmul(u, yc, ny) : cmac(P[j], u, yc, ny);
+        }
+      }
+      cneg2 nP[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) nP[j] = negated(P[j]);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const cdd2 x = pair_elements(__ldg(xu + i * v3), __ldg(xl + i * v1), kNeg1);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) A[i * 3 + j] = cmac(A[i * 3 + j], x, P[j], nP[j]);
+      }
+      yu += v1;
+      yl += v1;
+      xu += v1;
+      xl += v3;
+    }
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      if (!first_plane) {
+        const ulonglong2 sr = sum[(2 * e) * GF_NT], si = sum[(2 * e + 1) * GF_NT];
+        A[e] = {add(dd2{sr.x, sr.y}, A[e].re), add(dd2{si.x, si.y}, A[e].im)};
+      }
+      sum[(2 * e) * GF_NT] = make_ulonglong2(A[e].re.h, A[e].re.l);
+      sum[(2 * e + 1) * GF_NT] = make_ulonglong2(A[e].im.h, A[e].im.l);
+    }
+    first_plane = false;
   }
-  double *F = a.F + (size_t)(p * 4 + mu) * 8 * a.g.Vh + h;
+  Cx<df64> As[9], u1[9], t[9];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) F[(size_t)k * a.g.Vh] += f[k];
+  for (int k = 0; k < 9; ++k)
+    As[k] = {first(A[k].re) + second(A[k].re), first(A[k].im) + second(A[k].im)};
+  LinkIO<HMC_F64E, 18>::load(link_base<HMC_F64E, 18>(a.gauge, Vh, p, mu), Vh, h, u1);
+  m_mul(u1, As, t);
+  add_gauge_force<HMC_F64E, 18>(a, c, p, mu, h, u1, t);
 }
 
 // per site: sum_{mu<nu} Re Tr U_p and sum over extent-4 directions of s_mu Re Tr P_mu(x)
@@ -253,7 +373,10 @@ int gauge_force(hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, double beta, dou
     case HMC_F32 * 100 + 18: k_gauge_force<HMC_F32, 18><<<nb, 128, 0, strm>>>(a); break;
     case HMC_F32 * 100 + 12: k_gauge_force<HMC_F32, 12><<<nb, 128, 0, strm>>>(a); break;
     // emulated FP64: staples and U A in double-float, F accumulated in FP64
-    case HMC_F64E * 100 + 18: k_gauge_force<HMC_F64E, 18><<<nb, 128, 0, strm>>>(a); break;
+    case HMC_F64E * 100 + 18:
+      cudaFuncSetAttribute(k_gauge_force_e2, cudaFuncAttributeMaxDynamicSharedMemorySize, GF_SMEM);
+      k_gauge_force_e2<<<8 * blocks_for(g.Vh, GF_NT), GF_NT, GF_SMEM, strm>>>(a);
+      break;
     case HMC_F64E * 100 + 12: k_gauge_force<HMC_F64E, 12><<<nb, 128, 0, strm>>>(a); break;
     default: return fail(ctx, HMC_EINVAL, "gauge_force: links must be F64, F32 or F64E");
   }
