@@ -179,7 +179,7 @@ int hmc_ctx_set_timing(hmc_ctx *ctx, int enable);
 /* HMC_OPT_CG_GRAPH: 1 (default) runs every CG solve of hmc_cg_solve and
  * hmc_cg_solve_multi (and every solve inside the force, action and trajectory
  * calls) as one CUDA graph captured per solve: a while node over the loop body
- * (two iterations and a decision kernel), the reliable update in an if node,
+ * (two iterations, the second ending in the decision), the reliable update in an if node,
  * the convergence, reliable-update and iteration-limit decisions taken on the
  * device (for a batched solve: for all systems together), the host reading the
  * solver state once at the end.  The graph runs on a stream of the library's

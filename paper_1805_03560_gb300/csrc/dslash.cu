@@ -241,10 +241,10 @@ __device__ __forceinline__ void l2_prefetch(const void *p, unsigned bytes) {
 }
 
 template <int SP, int FMT>
-__device__ __forceinline__ void prefetch_block_links(const DslashArgs &a) {
+__device__ __forceinline__ void prefetch_block_links(const DslashArgs &a, int blk) {
   const int t = threadIdx.x;
   if (t >= 8) return;
-  const int Vh = a.g.Vh, h0 = ds_block(a) * DS_NT, mu = t >> 1;
+  const int Vh = a.g.Vh, h0 = blk * DS_NT, mu = t >> 1;
   const bool fwd = (t & 1) == 0;
   const int sh = fwd ? 0 : (mu == 3 ? 1 : a.g.st[mu] >> 1);
   int lo = h0 - sh, hi = h0 + DS_NT - sh + (!fwd && mu == 3 ? 1 : 0);
@@ -307,10 +307,9 @@ __device__ __forceinline__ void hops_rt(const DslashArgs &a, int h, int r, int l
 // Tiled (a.tile_nseg > 0, one right-hand side): the four warps of a block take
 // 32 consecutive sites each at the offsets {0, +x, +t, +x+t}, so half of the
 // x and t neighbours a block reads are its own sites and can hit in L1.
-__device__ __forceinline__ int dslash_site(const DslashArgs &a) {
-  if (a.tile_nseg == 0) return ds_block(a) * DS_NT + threadIdx.x;
+__device__ __forceinline__ int dslash_site(const DslashArgs &a, int b) {
+  if (a.tile_nseg == 0) return b * DS_NT + threadIdx.x;
   const int sx = a.g.L[2] * a.g.Lzh, st = a.g.L[1] * sx;
-  const int b = ds_block(a);
   const int seg = b % a.tile_nseg, xt = b / a.tile_nseg;
   const int hx = a.g.L[1] >> 1;
   const int xp = xt % hx, tp = xt / hx;
@@ -361,23 +360,33 @@ __global__ void __launch_bounds__(DS_NT, ds_min_blocks(SP, FMT, PAIR)) k_dslash(
   using R = typename SIO::R;
   constexpr int SF = DAG ? -1 : 1;  // forwards: 1 - gamma (1 + gamma for the adjoint)
   griddep_launch_dependents();
-  if constexpr ((SP == HMC_F32 || SP == HMC_F16 || SP == HMC_BF16) && FMT == 12)
-    if (a.prefetch) prefetch_block_links<SP, FMT>(a);  // links: not written by the kernel before
-  griddep_wait();
-  if (a.gate && *a.gate == 0) return;
   if (a.red_src && blockIdx.x == 0) {
+    // an extra block sums the partials of the launch before
+    griddep_wait();
+    if (a.gate && *a.gate == 0) return;
+    const double rr = a.red_alpha ? *a.red_rr : 0.0;
     const double t = block_sum_partials<DS_NT>(a.red_src, a.red_n);
     if (threadIdx.x == 0) {
       *a.red_dst = t;
       if (a.red_alpha) {
-        const double al = *a.red_rr / t;
+        const double al = rr / t;
         *a.red_alpha = al;
         if (!isfinite(al) || !(t > 0.0)) *a.red_flag = 2;
       }
     }
+    return;
   }
+  const int blk = ds_block(a, blockIdx.x - (a.red_src ? 1 : 0));
+  // the block's number for the end of the kernel, kept out of the registers
+  // the hops need
+  __shared__ int s_blk;
+  if (threadIdx.x == 0) s_blk = blk;
+  if constexpr ((SP == HMC_F32 || SP == HMC_F16 || SP == HMC_BF16) && FMT == 12)
+    if (a.prefetch) prefetch_block_links<SP, FMT>(a, blk);  // links: not written by the kernel before
+  griddep_wait();
+  if (a.gate && *a.gate == 0) return;
   const int S_ = a.g.Vh * a.n_rhs;
-  const int i = dslash_site(a);
+  const int i = dslash_site(a, blk);
   double nrm = 0.0;
   int r_out = -1;
   if (i < S_) {
@@ -423,28 +432,10 @@ __global__ void __launch_bounds__(DS_NT, ds_min_blocks(SP, FMT, PAIR)) k_dslash(
 #pragma unroll
       for (int k = 0; k < 12; ++k) acc[k] = cb * acc[k];
     }
-    if (a.cg_x) {
-      // fused CG step: acc = A p is consumed here, x += alpha p, r -= alpha A p
-      constexpr int PX = (SP == HMC_F64 || SP == HMC_F64E) ? SP : HMC_F32;
-      double ad;
-      if (a.cg_alpha) {
-        ad = *a.cg_alpha;  // formed once (and checked) by the launch before
-      } else {
-        const double pap = *a.cg_pap;
-        ad = *a.cg_rr / pap;
-        if (blockIdx.x == 0 && threadIdx.x == 0 && (!isfinite(ad) || !(pap > 0.0)))
-          *a.cg_flag = 2;
-      }
-      const R alpha = (R)ad;
-      Cx<R> pv[12], v[12];
-      SIO::load(a.cg_p, S_, i, pv);
-      load_as<PX>(a.cg_x, S_, i, v);
-#pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        v[k].re = fma(alpha, pv[k].re, v[k].re);
-        v[k].im = fma(alpha, pv[k].im, v[k].im);
-      }
-      store_as<PX>(a.cg_x, S_, i, v);
+    if (a.cg_r) {
+      // fused CG step: acc = A p is consumed here, r -= alpha A p
+      const R alpha = (R)*a.cg_alpha;  // formed (and checked) by the launch before
+      Cx<R> v[12];
       SIO::load(a.cg_r, S_, i, v);
 #pragma unroll
       for (int k = 0; k < 12; ++k) {
@@ -472,7 +463,7 @@ __global__ void __launch_bounds__(DS_NT, ds_min_blocks(SP, FMT, PAIR)) k_dslash(
   if (a.partials) {
     if (a.n_rhs == 1) {
       double s = block_sum<DS_NT>(nrm);
-      if (threadIdx.x == 0) a.partials[ds_block(a)] = s;
+      if (threadIdx.x == 0) a.partials[s_blk] = s;
       if (a.total) last_block_total<DS_NT>(a.partials, a.counter, a.total);
     } else {
       // one partial (and total) per right-hand side
@@ -483,8 +474,10 @@ __global__ void __launch_bounds__(DS_NT, ds_min_blocks(SP, FMT, PAIR)) k_dslash(
 }
 
 template <int SP, int FMT>
-static void launch_sf(const DslashArgs &a, int dagger, bool pair, int nb, cudaStream_t st) {
+static void launch_sf(DslashArgs a, int dagger, bool pair, int nb, cudaStream_t st) {
   const bool pdl = a.pdl != 0;
+  if (a.rev) a.rev = nb;
+  if (a.red_src) ++nb;
   if (pair) {
     if (dagger)
       launch_pdl(k_dslash<SP, FMT, true, true>, nb, DS_NT, st, pdl, a);
@@ -607,7 +600,7 @@ static int tune_variant(hmc_ctx *ctx, const DslashArgs &a, int sprec, int fmt, i
   const std::string key = tune_key(a, sprec, fmt, dagger);
   auto it = ctx->ds_tuned.find(key);
   if (it != ctx->ds_tuned.end()) return it->second;
-  const bool repeatable = !a.gate && !a.cg_x && !a.partials && !a.total && !a.red_src &&
+  const bool repeatable = !a.gate && !a.cg_r && !a.partials && !a.total && !a.red_src &&
                           a.out != a.x && a.out != a.in;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(ctx->stream, &cs);
@@ -679,11 +672,12 @@ int dslash(hmc_ctx *ctx, const DslashArgs &a, const hmc_gauge &U, int sprec, int
   // (BF16 storage: 2 bytes per real like F16, no norms)
   double bytes = (double)a.g.Vh * 8.0 * U.fmt * rb + (double)S * 24.0 * rb * (a.x ? 3.0 : 2.0);
   if (sprec == HMC_F16) bytes += (double)S * 4.0 * (a.x ? 3.0 : 2.0);
-  if (a.cg_x) {
-    // fused CG update: p, x, r read and x, r written, A p not written
-    const double xb = sprec == HMC_F64 ? 8.0 : 4.0;
-    bytes += (double)S * 24.0 * (3.0 * rb + 2.0 * xb - rb);
-    if (sprec == HMC_F16) bytes += (double)S * 4.0 * 2.0;
+  if (a.cg_r) {
+    // fused CG update: r read and written, A p not written (several systems:
+    // p and x read and x written too)
+    bytes += (double)S * 24.0 * rb;
+    if (sprec == HMC_F16) bytes += (double)S * 4.0;
+    if (a.cg_x) bytes += (double)S * 24.0 * (rb + 2.0 * 4.0);
   }
   char cls[64];
   snprintf(cls, sizeof(cls), "dslash_%s_%d%s%s",

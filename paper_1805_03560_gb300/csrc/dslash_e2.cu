@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(DS_NT, 3) k_dslash_e2(const DslashArgs a) {
   griddep_wait();
   if (a.gate && *a.gate == 0) return;
   const int Vh = a.g.Vh, S_ = Vh * a.n_rhs;
-  const int i = ds_block(a) * DS_NT + threadIdx.x;
+  const int blk = ds_block(a, blockIdx.x), i = blk * DS_NT + threadIdx.x;
   double nrm = 0.0;
   int r_out = -1;
   if (i < S_) {
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(DS_NT, 3) k_dslash_e2(const DslashArgs a) {
   if (a.partials) {
     if (a.n_rhs == 1) {
       const double t = block_sum<DS_NT>(nrm);
-      if (threadIdx.x == 0) a.partials[ds_block(a)] = t;
+      if (threadIdx.x == 0) a.partials[blk] = t;
       if (a.total) last_block_total<DS_NT>(a.partials, a.counter, a.total);
     } else {
       block_partials_rhs<DS_NT>(nrm, r_out, a.n_rhs, a.partials);
@@ -115,11 +115,12 @@ __global__ void __launch_bounds__(DS_NT, 3) k_dslash_e2(const DslashArgs a) {
 
 }  // namespace
 
-void launch_dslash_e2(const DslashArgs &a, int dagger, cudaStream_t st) {
+void launch_dslash_e2(DslashArgs a, int dagger, cudaStream_t st) {
+  const int nb = blocks_for((long long)a.g.Vh * a.n_rhs, DS_NT);
+  if (a.rev) a.rev = nb;
   const auto kernel = dagger ? k_dslash_e2<true> : k_dslash_e2<false>;
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, E2_SMEM);
-  launch_pdl_smem(kernel, blocks_for((long long)a.g.Vh * a.n_rhs, DS_NT), DS_NT, E2_SMEM, st,
-                  a.pdl != 0, a);
+  launch_pdl_smem(kernel, nb, DS_NT, E2_SMEM, st, a.pdl != 0, a);
 }
 
 }  // namespace hmc

@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(DS_NT, mr_min_blocks(NR)) k_dslash_mr(const Ds
   griddep_wait();
   if (a.gate && *a.gate == 0) return;
   const int n = a.n_rhs, NG = n / NR, St = a.g.Vh * n;
-  const int i = ds_block(a) * DS_NT + threadIdx.x;
+  const int i = ds_block(a, blockIdx.x) * DS_NT + threadIdx.x;
   double nrm[NR];
   int rr[NR];
 #pragma unroll
@@ -340,8 +340,9 @@ __global__ void __launch_bounds__(DS_NT, mr_min_blocks(NR)) k_dslash_mr(const Ds
 }
 
 template <int SP, int FMT, int NR>
-void launch_nr(const DslashArgs &a, int dagger, cudaStream_t st) {
+void launch_nr(DslashArgs a, int dagger, cudaStream_t st) {
   const int nb = blocks_for((long long)a.g.Vh * (a.n_rhs / NR), DS_NT);
+  if (a.rev) a.rev = nb;
   if (dagger)
     launch_pdl(k_dslash_mr<SP, FMT, true, NR>, nb, DS_NT, st, a.pdl != 0, a);
   else

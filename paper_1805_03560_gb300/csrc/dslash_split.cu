@@ -100,6 +100,22 @@ __global__ void __launch_bounds__(SPLIT_NT, split_min_blocks<SP>()) k_dslash_spl
   griddep_launch_dependents();
   const int mu = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int Vh = a.g.Vh;
+  if (a.red_src && blockIdx.x == gridDim.x - 1) {
+    // the block after the lattice's: sum the partials of the launch before
+    griddep_wait();
+    if (a.gate && *a.gate == 0) return;
+    const double rr = a.red_alpha ? *a.red_rr : 0.0;
+    const double t = block_sum_partials<SPLIT_NT>(a.red_src, a.red_n);
+    if (threadIdx.x == 0) {
+      *a.red_dst = t;
+      if (a.red_alpha) {
+        const double al = rr / t;
+        *a.red_alpha = al;
+        if (!isfinite(al) || !(t > 0.0)) *a.red_flag = 2;
+      }
+    }
+    return;
+  }
   const int i = blockIdx.x * SPLIT_SITES + lane;
   const bool in = i < Vh;
   const int is = in ? i : Vh - 1;  // threads past the end work on the last site and store nothing
@@ -112,6 +128,20 @@ __global__ void __launch_bounds__(SPLIT_NT, split_min_blocks<SP>()) k_dslash_spl
   const bool wf = mu == 0 && cm + 1 == Lm, wb = mu == 0 && cm == 0;
   const void *gf = link_base<SP, FMT>(a.gauge, Vh, a.p, mu);
   const void *gb = link_base<SP, FMT>(a.gauge, Vh, 1 - a.p, mu);
+  // loads that depend on nothing computed here are issued before the gate is
+  // looked at and before the hops: the epilogue's fields, the factor alpha
+  constexpr int NE = (NCH + 3) / 4;  // chunks per thread in the epilogue
+  constexpr bool EARLY = SP == HMC_F32;
+  Cx<R> xe[NE][CPC], re[NE][CPC];
+  const auto load_epilogue = [&] {
+#pragma unroll
+    for (int e = 0; e < NE; ++e)
+      if (mu + 4 * e < NCH) {
+        if (a.x) CIO::load(a.x, Vh, mu + 4 * e, is, xe[e]);
+        if (a.cg_r) CIO::load(a.cg_r, Vh, mu + 4 * e, is, re[e]);
+      }
+  };
+  double alpha_d = 0.0;
   Cx<R> acc[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = {R(0), R(0)};
@@ -152,9 +182,12 @@ __global__ void __launch_bounds__(SPLIT_NT, split_min_blocks<SP>()) k_dslash_spl
     LIO::load(gf, Vh, is, uf);
     LIO::load(gb, Vh, hb, ub);
     if (a.links_ready) griddep_wait();
-    if (a.gate && *a.gate == 0) return;
+    const int live = a.gate ? *a.gate : 1;
     SIO::load(a.in, Vh, hf, pf);
     SIO::load(a.in, Vh, hb, pb);
+    if (a.cg_r) alpha_d = *a.cg_alpha;
+    if constexpr (EARLY) load_epilogue();
+    if (!live) return;
     project_mu<SF>(mu, pf, hs);
     flip(wf, hs);
     mul_link(uf, hs, w);
@@ -164,68 +197,47 @@ __global__ void __launch_bounds__(SPLIT_NT, split_min_blocks<SP>()) k_dslash_spl
     mul_link_dag(ub, hs, w);
     accumulate_mu<-SF>(mu, acc, w);
   }
-  if (a.red_src && blockIdx.x == 0) {
-    const double t = block_sum_partials<SPLIT_NT>(a.red_src, a.red_n);
-    if (threadIdx.x == 0) {
-      *a.red_dst = t;
-      if (a.red_alpha) {
-        const double al = *a.red_rr / t;
-        *a.red_alpha = al;
-        if (!isfinite(al) || !(t > 0.0)) *a.red_flag = 2;
-      }
-    }
-  }
 #pragma unroll
   for (int k = 0; k < NCH; ++k)
 #pragma unroll
     for (int j = 0; j < CPC; ++j) s_w[mu][k][lane][j] = acc[k * CPC + j];
+  if constexpr (!EARLY) load_epilogue();
   __syncthreads();
   R n2 = R(0);
   if (in) {
-    const R cb = (R)a.cb, ca = (R)a.ca;
-    const R alpha = a.cg_x ? (R)*a.cg_alpha : R(0);
+    const R cb = (R)a.cb, ca = (R)a.ca, alpha = (R)alpha_d;
 #pragma unroll
-    for (int ch = mu; ch < NCH; ch += 4) {
-      Cx<R> t[CPC], v[CPC];
+    for (int e = 0; e < NE; ++e) {
+      const int ch = mu + 4 * e;
+      if (ch >= NCH) break;
+      Cx<R> t[CPC];
 #pragma unroll
       for (int j = 0; j < CPC; ++j)
         t[j] = ((s_w[0][ch][lane][j] + s_w[1][ch][lane][j]) + s_w[2][ch][lane][j]) +
                s_w[3][ch][lane][j];
       if (a.x) {
-        CIO::load(a.x, Vh, ch, i, v);
 #pragma unroll
         for (int j = 0; j < CPC; ++j) {
-          t[j].re = fma(ca, v[j].re, cb * t[j].re);
-          t[j].im = fma(ca, v[j].im, cb * t[j].im);
+          t[j].re = fma(ca, xe[e][j].re, cb * t[j].re);
+          t[j].im = fma(ca, xe[e][j].im, cb * t[j].im);
         }
       } else {
 #pragma unroll
         for (int j = 0; j < CPC; ++j) t[j] = cb * t[j];
       }
-      if (a.cg_x) {
-        // fused CG step: x += alpha p, r -= alpha A p (A p = t is not stored)
-        Cx<R> pv[CPC];
-        CIO::load(a.cg_p, Vh, ch, i, pv);
-        CIO::load(a.cg_x, Vh, ch, i, v);
+      if (a.cg_r) {
+        // fused CG step: r -= alpha A p (A p = t is not stored)
 #pragma unroll
         for (int j = 0; j < CPC; ++j) {
-          v[j].re = fma(alpha, pv[j].re, v[j].re);
-          v[j].im = fma(alpha, pv[j].im, v[j].im);
+          t[j].re = fma(-alpha, t[j].re, re[e][j].re);
+          t[j].im = fma(-alpha, t[j].im, re[e][j].im);
         }
-        CIO::store(a.cg_x, Vh, ch, i, v);
-        CIO::load(a.cg_r, Vh, ch, i, v);
-#pragma unroll
-        for (int j = 0; j < CPC; ++j) {
-          v[j].re = fma(-alpha, t[j].re, v[j].re);
-          v[j].im = fma(-alpha, t[j].im, v[j].im);
-          n2 += norm2(v[j]);
-        }
-        CIO::store(a.cg_r, Vh, ch, i, v);
+        CIO::store(a.cg_r, Vh, ch, i, t);
       } else {
         CIO::store(a.out, Vh, ch, i, t);
-#pragma unroll
-        for (int j = 0; j < CPC; ++j) n2 += norm2(t[j]);
       }
+#pragma unroll
+      for (int j = 0; j < CPC; ++j) n2 += norm2(t[j]);
     }
   }
   if (a.partials) {
@@ -245,7 +257,7 @@ __global__ void __launch_bounds__(SPLIT_NT, split_min_blocks<SP>()) k_dslash_spl
 
 template <int SP, int FMT>
 void launch_fmt(const DslashArgs &a, int dagger, cudaStream_t st) {
-  const int nb = blocks_for(a.g.Vh, SPLIT_SITES);
+  const int nb = blocks_for(a.g.Vh, SPLIT_SITES) + (a.red_src ? 1 : 0);
   if (dagger)
     launch_pdl(k_dslash_split<SP, FMT, true>, nb, SPLIT_NT, st, a.pdl != 0, a);
   else
@@ -266,10 +278,9 @@ int dslash_split_blocks(const Geo &g) { return blocks_for(g.Vh, SPLIT_SITES); }
 //   FP64 (bound by its pipe, 25 % dearer per site here), per CG iteration:
 //     20736 282 / 208 us, 36864 285 / 319, 65536 550 / 549, 128000 953 / 1034:
 //     where the fullest SM gets enough fewer sites.
-// The fused CG update needs alpha formed by the launch before; per-right-
-// hand-side factors belong to several right-hand sides.
+// Per-right-hand-side factors belong to several right-hand sides.
 bool dslash_split_rule(const hmc_ctx *ctx, const DslashArgs &a, int sprec) {
-  if (a.n_rhs != 1 || a.cb_rhs || (a.cg_x && !a.cg_alpha)) return false;
+  if (a.n_rhs != 1 || a.cb_rhs) return false;
   const long long Vh = a.g.Vh, sms = ctx->sm_count;
   switch (sprec) {
     case HMC_F32: return Vh <= 256 * sms;

@@ -170,34 +170,28 @@ struct DslashArgs {
   // zeroed device int, returned to zero)
   double *total;
   unsigned int *counter;
-  // before its stencil work, block 0 sums red_src[0..red_n) (the block
-  // partials a previous launch left) in a fixed order into *red_dst
+  // one more block sums red_src[0..red_n) (the block partials a previous
+  // launch left) in a fixed order into *red_dst
   const double *red_src;
   int red_n;
   double *red_dst;
-  // with red_alpha: block 0 also stores *red_alpha = *red_rr / (the sum),
+  // with red_alpha: it also stores *red_alpha = *red_rr / (the sum),
   // *red_flag = 2 when that is not finite or the sum is not positive
   const double *red_rr;
   double *red_alpha;
   int *red_flag;
-  // fused CG update (n_rhs == 1): the epilogue result A p is not stored;
-  // with alpha = *cg_rr / *cg_pap the launch updates x += alpha p (cg_x, in
-  // FP64 for FP64 fields, F32 otherwise) and r -= alpha A p (cg_r), and the
-  // partials receive |r|^2.  *cg_flag = 2 when alpha is not finite.
-  void *cg_x;
+  // fused CG update (n_rhs == 1): the epilogue result A p is not stored; with
+  // alpha = *cg_alpha (formed by an earlier launch, red_alpha) the launch
+  // updates r -= alpha A p (cg_r) and the partials receive |r|^2
   void *cg_r;
-  const void *cg_p;
-  const double *cg_rr;
-  const double *cg_pap;
-  int *cg_flag;
-  // nullable: alpha precomputed by an earlier launch (red_alpha); the fused
-  // update then reads it instead of dividing cg_rr by cg_pap
   const double *cg_alpha;
   // fused update of the batched CG (n_rhs > 1, multi-right-hand-side
   // kernel only): per system alpha_r = mcg_rr[r] / mcg_pap[r] when
   // mcg_live[r] (0 otherwise; mcg_done[r] = 2 when not finite), x_r +=
-  // alpha_r p_r (cg_x in F32), r_r -= alpha_r A p_r (cg_r), |r_r|^2
+  // alpha_r p_r (cg_x in F32, cg_p), r_r -= alpha_r A p_r (cg_r), |r_r|^2
   // partials and totals (partials, total, counter)
+  void *cg_x;
+  const void *cg_p;
   const double *mcg_rr;
   const double *mcg_pap;
   const int *mcg_live;
@@ -209,7 +203,9 @@ struct DslashArgs {
   // solve): the one-thread-per-direction kernel may load them before its wait for
   // the launch before
   int links_ready;
-  int rev;  // set by dslash(): walk the lattice from its last block to its first
+  // walk the lattice from its last block to its first: a flag set by dslash(),
+  // the number of lattice blocks in the kernels (set by the launchers)
+  int rev;
 };
 // Block of the lattice this thread block works on.  Consecutive launches of a
 // chain of hemi-Dslashes read the same links and each other's output; on a
@@ -220,12 +216,13 @@ struct DslashArgs {
 // FP32 and 174.3 -> 166.8 us in F16, on 32^3 x 64 582.9 -> 563.4 us; no
 // difference where the fields fit in L2.  Results do not depend on it: a
 // block's partial sum is stored under the lattice block it belongs to.
-__device__ __forceinline__ int ds_block(const DslashArgs &a) {
-  return a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+// b: the block's number among those that work on the lattice.
+__device__ __forceinline__ int ds_block(const DslashArgs &a, int b) {
+  return a.rev ? a.rev - 1 - b : b;
 }
 // Emulated FP64 with 18-real links, one thread per site and right-hand side
 // (dslash_e2.cu)
-void launch_dslash_e2(const DslashArgs &a, int dagger, cudaStream_t st);
+void launch_dslash_e2(DslashArgs a, int dagger, cudaStream_t st);
 // One-thread-per-direction hemi-Dslash (dslash_split.cu) of one right-hand
 // side: whether it is the kernel for this launch, its launch, and its block
 // count (the partials it leaves; the kernels of DS_NT threads leave fewer).

@@ -2,18 +2,20 @@
 // with BiCGstab to machine precision, Sec. IV, the solution is the same).
 //
 // One iteration is five launches (one_iteration): the two hemi-Dslash of
-// y = Mhat p (the second leaves block partials of |y|^2 = p^dag A p), the
-// two of Mhat^dag y (the first also sums those partials into pap in its
-// block 0; the second consumes A p in its epilogue: alpha = rr / pap,
-// x += alpha p, r -= alpha A p, block partials of |r|^2), then xpay
-// (every block sums those in one fixed order: beta = |r|^2 / rr,
-// p = r + beta p).  No reduction needs a kernel of its own, a grid-wide
-// fence or an atomic.  rr is double-buffered
-// by iteration parity (passed by the host, which knows the iteration it
-// enqueues), so block 0 can store the new value while other blocks still read
-// the old one.  Scalars never leave the device during a batch of iterations;
-// the host reads the state once per batch, sizing the next batch from the
-// observed convergence rate.
+// y = Mhat p (the second leaves block partials of |y|^2 = p^dag A p), the two
+// of Mhat^dag y (an extra block of the first sums those partials into pap and
+// forms alpha = rr / pap; the second consumes A p in its epilogue,
+// r -= alpha A p, and leaves block partials of |r|^2), then xpay (every block
+// sums those in one fixed order: beta = |r|^2 / rr, x += alpha p,
+// p = r + beta p; the x update sits there because p is read there anyway).  No
+// reduction needs a kernel of its own, a grid-wide fence or an atomic, and the
+// decision after every second iteration is taken by xpay's block 0.  rr is
+// double-buffered by iteration parity (passed by the host, which knows the
+// iteration it enqueues), so block 0 can store the new value while other blocks
+// still read the old one.
+// Measured (x in the fused hemi-Dslash, a decision kernel, block 0 summing
+// besides its stencil -> this form), per iteration: 8^3 x 16 23.2 -> 20.9 us,
+// 12^3 x 24 30.8 -> 28.4 us, 24^3 x 48 187.3 -> 184.3 us.
 //
 // Plain FP64: textbook CG on FP64 fields; xpay raises `done` when the
 // recursive residual reaches the tolerance and the host confirms it on the
@@ -27,6 +29,7 @@
 // fixed order, so solves are bit-reproducible.
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "hmc_host.h"
 
@@ -40,10 +43,13 @@ struct CGState {
   double rr_next; // |r|^2 after the update (set by xpay)
   double alpha;   // rr / pap of the current iteration (block 0 of the H_eo^dag launch)
   int done;       // 1 converged (recursive residual), 2 NaN/Inf
-  int active;     // !done
+  // gate[par]: the launches of an iteration of parity par run; xpay of parity
+  // par sets the other one (it may stop the solve while blocks of its own
+  // launch still look at gate[par])
+  int gate[2];
   int iter;
-  int iter_cap;   // xpay clears `active` once iter reaches it
-  // iteration control on the device (k_cg_control_init, k_cg_decide, k_cg_ru_end)
+  int iter_cap;   // xpay stops the iterations once iter reaches it
+  // iteration control on the device (k_cg_control_init, cg_decide, k_cg_ru_end)
   double thr;     // tol^2 |b|^2
   double maxr2;   // largest |r|^2 since the last reliable update
   double delta2;  // reliable-update threshold delta^2
@@ -156,75 +162,171 @@ __global__ void __launch_bounds__(BL_NT) k_dot(const void *x, const void *y, int
 // on 24^3 x 48 this beats one block summing them in a kernel of its own, and
 // a sum with more loads in flight per thread: all blocks read the same few
 // L2 lines at once.)
+__device__ void cg_decide(CGState *st, cudaGraphConditionalHandle upd,
+                          cudaGraphConditionalHandle loop, int in_graph);
+
+// Sum of the partials by one block, beta, and (block 0) the state: the part of
+// xpay that precedes its update.  `gate`, `rr_old`: the state as read at the
+// start of the kernel.
+template <int NT, typename R>
+__device__ __forceinline__ void xpay_head(CGState *st, int gate, double rr_old, int par, int plain,
+                                          const double *rr_part, int n_part,
+                                          cudaGraphConditionalHandle upd,
+                                          cudaGraphConditionalHandle loop, int in_graph,
+                                          R *s_beta) {
+  __shared__ double s_part[NT / 32];
+  double t = 0.0;
+  for (int j = threadIdx.x; j < n_part; j += NT) t += __ldcg(rr_part + j);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    t = threadIdx.x < NT / 32 ? s_part[threadIdx.x] : 0.0;
+#pragma unroll
+    for (int o = NT / 64; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  }
+  if (threadIdx.x == 0) {
+    *s_beta = (R)(t / rr_old);
+    if (blockIdx.x == 0) {
+      int on = gate;
+      if (gate) {
+        st->rr_next = t;
+        st->rr[par ^ 1] = t;
+        st->iter += 1;
+        if (!isfinite(t) || st->done == 2) {
+          st->done = 2;
+          on = 0;
+        } else if (plain && t <= st->tol2 * st->b2) {
+          st->done = 1;
+          on = 0;
+        }
+        if (st->iter >= st->iter_cap) on = 0;
+      }
+      st->gate[par ^ 1] = on;
+      // the second iteration of a pair ends with the decision
+      if (par) cg_decide(st, upd, loop, in_graph);
+    }
+  }
+  __syncthreads();
+}
+
+// FP32 and FP64: the fields are the same sequence of 16-byte chunks, one chunk
+// per thread and pass.  What bounds it is memory (five streams); many light
+// threads keep it busy where one thread per site (twelve components of three
+// fields in registers, two blocks per SM) left it with a nearly empty last
+// pass: a CG iteration on 24^3 x 48 199 us with that form.
+constexpr int XP_NT = 512;
+constexpr int XP_BLOCKS = 3;  // per SM
+
+__device__ __forceinline__ float4 axpy4(float a, float4 x, float4 y) {
+  return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
+}
+__device__ __forceinline__ double2 axpy4(double a, double2 x, double2 y) {
+  return make_double2(fma(a, x.x, y.x), fma(a, x.y, y.y));
+}
+
 template <int PL>
-__global__ void __launch_bounds__(BL_NT) k_cg_xpay(void *p, const void *r, int S, CGState *st,
-                                                   int par, int plain, const double *rr_part,
-                                                   int n_part, int rev) {
+__global__ void __launch_bounds__(XP_NT, XP_BLOCKS) k_cg_xpay_chunks(
+    void *x, void *p, const void *r, int S, CGState *st, int par, int plain, const double *rr_part,
+    int n_part, int rev, cudaGraphConditionalHandle upd, cudaGraphConditionalHandle loop,
+    int in_graph) {
+  using R = RT<PL>;
+  using V = std::conditional_t<PL == HMC_F32, float4, double2>;
   griddep_launch_dependents();
   griddep_wait();
-  if (!st->active) return;
-  using R = RT<PL>;
-  // the first grid-stride element's r and p are loaded before the sum of the
-  // partials, so that their DRAM latency overlaps the reduction
+  // everything this thread needs first is asked for at once
+  const int gate = st->gate[par];
+  const R alpha = (R)st->alpha;
+  const double rr_old = st->rr[par];
+  V *xf = (V *)x, *pf = (V *)p;
+  const V *rf = (const V *)r;
+  // chunks, in groups of 32 threads on 32 consecutive ones; in FP32 a group is
+  // one chunk plane of a block of 32 sites, partly past the end in the last block
+  const long long n = PL == HMC_F32 ? (long long)f32_sites(S) * 6 : ((long long)S * 12 + 31) & ~31LL;
+  const long long stride = (long long)gridDim.x * XP_NT;
+  // rev: from the last chunk to the first (the launch before, the fused update,
+  // went the other way and left its last elements in L2)
+  const auto at = [&](long long j) { return rev ? n - 1 - j : j; };
+  const auto valid = [&](long long c) {
+    if (PL == HMC_F32) return (c / 192) * 32 + (c & 31) < S;
+    return c < (long long)S * 12;
+  };
+  long long j = (long long)blockIdx.x * XP_NT + threadIdx.x;
+  V xv, pv, rv;
+  const auto load = [&](long long c) {
+    rv = rf[c];
+    pv = pf[c];
+    xv = xf[c];
+  };
+  bool on = j < n && valid(at(j));
+  if (on) load(at(j));
+  __shared__ R s_beta;
+  xpay_head<XP_NT, R>(st, gate, rr_old, par, plain, rr_part, n_part, upd, loop, in_graph, &s_beta);
+  if (!gate) return;
+  const R beta = s_beta;
+  while (j < n) {
+    if (on) {
+      const long long c = at(j);
+      xf[c] = axpy4(alpha, pv, xv);
+      pf[c] = axpy4(beta, pv, rv);
+    }
+    j += stride;
+    on = j < n && valid(at(j));
+    if (on) load(at(j));
+  }
+}
+
+// half storage: one thread per site (F16: the norm needs the whole site)
+template <int PL>
+__global__ void __launch_bounds__(BL_NT) k_cg_xpay(void *x, void *p, const void *r, int S,
+                                                   CGState *st, int par, int plain,
+                                                   const double *rr_part, int n_part, int rev,
+                                                   cudaGraphConditionalHandle upd,
+                                                   cudaGraphConditionalHandle loop,
+                                                   int in_graph) {
+  griddep_launch_dependents();
+  griddep_wait();
+  // everything this thread needs first is asked for at once: the state, the
+  // first grid-stride element of x, r and p, the partials
+  const int gate = st->gate[par];
+  const float alpha = (float)st->alpha;
+  const double rr_old = st->rr[par];
   const int j0 = blockIdx.x * BL_NT + threadIdx.x;
-  // rev: from the last element to the first (the launch before, the fused
-  // update, went the other way and left its last elements in L2); top makes
-  // groups of 32 consecutive threads whole groups of 32 elements
   const int top = ((S + 31) & ~31) - 1;
   const auto at = [&](int j) { return rev ? top - j : j; };
-  const int i0 = at(j0);
-  Cx<R> rv[12], pv[12];
-  if (j0 <= top && i0 < S) {
-    load_as<PL>(r, S, i0, rv);
-    load_as<PL>(p, S, i0, pv);
-  }
-  __shared__ double s_rr;
-  {
-    double t = 0.0;
-    for (int j = threadIdx.x; j < n_part; j += BL_NT) t += __ldcg(rr_part + j);
-    t = block_sum<BL_NT>(t);
-    if (threadIdx.x == 0) s_rr = t;
-  }
-  __syncthreads();  // every thread has the sum and has read the state before block 0 updates it
-  const double rr_new = s_rr;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    st->rr_next = rr_new;
-    st->rr[par ^ 1] = rr_new;
-    st->iter += 1;
-    if (!isfinite(rr_new) || st->done == 2) {
-      st->done = 2;
-      st->active = 0;
-    } else if (plain && rr_new <= st->tol2 * st->b2) {
-      st->done = 1;
-      st->active = 0;
+  Cx<float> rv[12], pv[12], xv[12];
+  const auto load = [&](int j) {
+    const int i = at(j);
+    if (j <= top && i < S) {
+      load_as<PL>(r, S, i, rv);
+      load_as<PL>(p, S, i, pv);
+      load_as<HMC_F32>(x, S, i, xv);
     }
-    if (st->iter >= st->iter_cap) st->active = 0;
-  }
-  const R beta = (R)(rr_new / st->rr[par]);
+  };
+  load(j0);
+  __shared__ float s_beta;
+  xpay_head<BL_NT, float>(st, gate, rr_old, par, plain, rr_part, n_part, upd, loop, in_graph,
+                          &s_beta);
+  if (!gate) return;
+  const float beta = s_beta;
   // grid-stride: the grid is a few blocks per SM, so few blocks read the
-  // partials; the next element's loads are issued before the current one is
-  // updated, two elements in flight per thread
+  // partials
   const int stride = gridDim.x * BL_NT;
   for (int j = j0; j <= top; j += stride) {
-    Cx<R> rn[12], pn[12];
-    const int i = at(j), in = at(j + stride);
-    if (j + stride <= top && in < S) {
-      load_as<PL>(r, S, in, rn);
-      load_as<PL>(p, S, in, pn);
-    }
+    const int i = at(j);
     if (i < S) {
 #pragma unroll
       for (int k = 0; k < 12; ++k) {
+        xv[k].re = fma(alpha, pv[k].re, xv[k].re);
+        xv[k].im = fma(alpha, pv[k].im, xv[k].im);
         pv[k].re = fma(beta, pv[k].re, rv[k].re);
         pv[k].im = fma(beta, pv[k].im, rv[k].im);
       }
+      store_as<HMC_F32>(x, S, i, xv);
       store_as<PL>(p, S, i, pv);
     }
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      rv[k] = rn[k];
-      pv[k] = pn[k];
-    }
+    load(j + stride);
   }
 }
 
@@ -281,13 +383,13 @@ __global__ void __launch_bounds__(FIN_NT) k_cg_init(CGState *st, const double *p
     st->iter = 0;
     st->iter_cap = 0x7fffffff;
     st->done = (s == 0.0) ? 1 : (isfinite(s) ? 0 : 2);
-    st->active = st->done == 0;
+    st->gate[0] = st->gate[1] = st->done == 0;
   }
 }
 
 // ---- iteration control on the device ----------------------------------------------
 // A solve is a loop of bodies: two iterations (parities 0 and 1), then
-// k_cg_decide.  When that asks for a reliable update (mixed precision: |r|^2
+// cg_decide.  When that asks for a reliable update (mixed precision: |r|^2
 // below the tolerance or below delta^2 times its largest value since the
 // last update) or for a true-residual check (plain FP64: the recursive
 // residual has converged), the update follows: fold the low-precision iterate
@@ -312,21 +414,22 @@ __global__ void k_cg_control_init(CGState *st, double delta2, int max_iter, int 
   st->bodies = 0;
   st->max_bodies = max_bodies;
   st->stop = st->done == 1 ? 1 : (st->done == 2 ? 2 : (max_iter > 0 ? 0 : 3));
-  if (st->stop) st->active = 0;
+  if (st->stop) st->gate[0] = st->gate[1] = 0;
 }
 
-// after each pair of iterations: NaN, a pending reliable update or check, the
-// iteration limit.  In a graph, `upd` receives whether the update runs and
-// `loop` whether the loop goes on: it does while the solve runs (after an
+// After each pair of iterations (one thread, at the end of the second xpay):
+// NaN, a pending reliable update or check, the iteration limit; gate[0] opens
+// or closes the next pair.  In a graph, `upd` receives whether the update runs
+// and `loop` whether the loop goes on: it does while the solve runs (after an
 // update that stops it, the next body's launches are gated off and its
 // decision ends the loop), within the body bound.
-__global__ void k_cg_decide(CGState *st, cudaGraphConditionalHandle upd,
-                            cudaGraphConditionalHandle loop, int in_graph) {
+__device__ void cg_decide(CGState *st, cudaGraphConditionalHandle upd,
+                          cudaGraphConditionalHandle loop, int in_graph) {
   int ru = 0;
   if (st->stop == 0) {
     if (st->done == 2) {
       st->stop = 2;
-      st->active = 0;
+      st->gate[0] = 0;
     } else if (!st->mixed) {
       ru = st->done == 1;
     } else {
@@ -336,10 +439,10 @@ __global__ void k_cg_decide(CGState *st, cudaGraphConditionalHandle upd,
     }
     if (!ru && st->stop == 0 && st->iter >= st->max_iter) {
       st->stop = 3;
-      st->active = 0;
+      st->gate[0] = 0;
     }
   }
-  if (ru) st->active = 0;
+  if (ru) st->gate[0] = 0;
   st->ru = ru;
   st->bodies += 1;
   if (in_graph) {
@@ -364,17 +467,17 @@ __global__ void __launch_bounds__(FIN_NT) k_cg_ru_end(CGState *st, const double 
     st->restarts += 1;
   if (!isfinite(s)) {
     st->done = 2;
-    st->active = 0;
+    st->gate[0] = 0;
     st->stop = 2;
   } else if (s <= st->thr) {
-    st->active = 0;
+    st->gate[0] = 0;
     st->stop = 1;
   } else if ((!st->mixed && st->restarts > 5) || st->iter >= st->max_iter) {
-    st->active = 0;
+    st->gate[0] = 0;
     st->stop = 3;
   } else {
     st->done = 0;
-    st->active = 1;
+    st->gate[0] = 1;
   }
 }
 
@@ -390,10 +493,10 @@ __global__ void __launch_bounds__(FIN_NT) k_cg_restart(CGState *st, const double
     st->aux = s;
     if (!isfinite(s)) {
       st->done = 2;
-      st->active = 0;
+      st->gate[0] = 0;
     } else {
       st->done = 0;
-      st->active = 1;
+      st->gate[0] = 1;
     }
   }
 }
@@ -501,22 +604,38 @@ int apply_A64(Solve &s, const void *in, void *out) {
   return hi_mdagm(s.hi, out, in, s.kappa, 1, nullptr);
 }
 
+// handles of the graph's conditional nodes (0 outside a graph)
+struct Handles {
+  cudaGraphConditionalHandle upd = 0, loop = 0;
+  int in_graph = 0;
+};
+
 template <int PL>
-void launch_xpay(Solve &s, int par, int n_part) {
-  const int nb = s.nb_bl < 2 * s.ctx->sm_count ? s.nb_bl : 2 * s.ctx->sm_count;
-  launch_pdl(k_cg_xpay<PL>, nb, BL_NT, s.ctx->stream, s.ctx->pdl != 0, s.p, (const void *)s.rlo,
-             s.S, s.st, par, s.plo == HMC_F64 ? 1 : 0, (const double *)s.rr_part, n_part,
-             s.ctx->ds_rev ^= 1);
+void launch_xpay(Solve &s, int par, int n_part, const Handles &h) {
+  const int plain = s.plo == HMC_F64 ? 1 : 0, rev = s.ctx->ds_rev ^= 1;
+  void *x = plain ? s.x : s.xlo;
+  if constexpr (PL == HMC_F32 || PL == HMC_F64) {
+    const long long n = PL == HMC_F32 ? (long long)f32_sites(s.S) * 6 : (long long)s.S * 12;
+    const int all = blocks_for(n, XP_NT), most = XP_BLOCKS * s.ctx->sm_count;
+    launch_pdl(k_cg_xpay_chunks<PL>, all < most ? all : most, XP_NT, s.ctx->stream,
+               s.ctx->pdl != 0, x, s.p, (const void *)s.rlo, s.S, s.st, par, plain,
+               (const double *)s.rr_part, n_part, rev, h.upd, h.loop, h.in_graph);
+  } else {
+    const int nb = s.nb_bl < 2 * s.ctx->sm_count ? s.nb_bl : 2 * s.ctx->sm_count;
+    launch_pdl(k_cg_xpay<PL>, nb, BL_NT, s.ctx->stream, s.ctx->pdl != 0, x, s.p,
+               (const void *)s.rlo, s.S, s.st, par, plain, (const double *)s.rr_part, n_part, rev,
+               h.upd, h.loop, h.in_graph);
+  }
 }
 
 // One iteration, five launches: y = Mhat p (the second hemi-Dslash leaves
-// block partials of |y|^2 = p^dag A p), t = H_eo^dag y (its block 0 sums
+// block partials of |y|^2 = p^dag A p), t = H_eo^dag y (an extra block sums
 // those partials into pap and forms alpha = rr / pap once), then the second
-// hemi-Dslash of Mhat^dag with the fused update x += alpha p,
-// r -= alpha A p (A p is never stored; it leaves
-// block partials of |r|^2), then xpay (every block sums the |r|^2 partials:
-// beta = |r|^2 / rr; p = r + beta p; block 0 advances the state).
-int one_iteration(Solve &s, int k) {
+// hemi-Dslash of Mhat^dag with the fused update r -= alpha A p (A p is never
+// stored; it leaves block partials of |r|^2), then xpay (every block sums the
+// |r|^2 partials: beta = |r|^2 / rr; x += alpha p; p = r + beta p; block 0
+// advances the state and, after the second iteration of a pair, decides).
+int one_iteration(Solve &s, int k, const Handles &h = Handles()) {
   hmc_ctx *ctx = s.ctx;
   const bool mixed = s.plo != HMC_F64;
   const hmc_gauge &U = mixed ? s.Ul : s.Uh;
@@ -525,7 +644,7 @@ int one_iteration(Solve &s, int k) {
   a.g = s.g;
   a.n_rhs = 1;
   a.gauge = U.data;
-  a.gate = &s.st->active;
+  a.gate = &s.st->gate[par];
   a.tag = "cg";
   a.links_ready = 1;
   // t = H_oe p; y = p - kappa^2 H_eo t with |y|^2 block partials
@@ -545,21 +664,16 @@ int one_iteration(Solve &s, int k) {
   a.red_rr = nullptr; a.red_alpha = nullptr; a.red_flag = nullptr;
   // A p = y - kappa^2 H_oe^dag t consumed by the fused update
   a.p = 0; a.out = nullptr; a.in = s.tlo; a.x = s.y; a.ca = 1.0; a.cb = -s.kappa * s.kappa;
-  a.cg_x = mixed ? s.xlo : s.x;
   a.cg_r = s.rlo;
-  a.cg_p = s.p;
-  a.cg_rr = &s.st->rr[par];
-  a.cg_pap = &s.st->pap;
-  a.cg_flag = &s.st->done;
   a.cg_alpha = &s.st->alpha;
   a.partials = s.rr_part;
   int nb_rr = 0;
   TRY(dslash(ctx, a, U, s.plo, 1, &nb_rr));
   switch (s.plo) {
-    case HMC_F64: launch_xpay<HMC_F64>(s, par, nb_rr); break;
-    case HMC_F32: launch_xpay<HMC_F32>(s, par, nb_rr); break;
-    case HMC_F16: launch_xpay<HMC_F16>(s, par, nb_rr); break;
-    case HMC_BF16: launch_xpay<HMC_BF16>(s, par, nb_rr); break;
+    case HMC_F64: launch_xpay<HMC_F64>(s, par, nb_rr, h); break;
+    case HMC_F32: launch_xpay<HMC_F32>(s, par, nb_rr, h); break;
+    case HMC_F16: launch_xpay<HMC_F16>(s, par, nb_rr, h); break;
+    case HMC_BF16: launch_xpay<HMC_BF16>(s, par, nb_rr, h); break;
   }
   return launched(ctx, "cg_xpay");
 }
@@ -613,12 +727,10 @@ int true_residual_restart(Solve &s, int par, bool restart_lo, double *rr) {
   return 0;
 }
 
-// the loop body: two iterations and the decision (`handle` receives it in a graph)
-int body_pair(Solve &s, cudaGraphConditionalHandle handle, int in_graph) {
+// the loop body: two iterations, the second ending in the decision
+int body_pair(Solve &s) {
   TRY(one_iteration(s, 0));
-  TRY(one_iteration(s, 1));
-  k_cg_decide<<<1, 1, 0, s.ctx->stream>>>(s.st, handle, 0, in_graph);
-  return launched(s.ctx, "cg_decide");
+  return one_iteration(s, 1);
 }
 
 // the reliable update (plain CG: the true-residual check and restart)
@@ -633,15 +745,17 @@ int body_update(Solve &s) {
 }
 
 // ---- the whole solve as one CUDA graph (capture_loop) -----------------------------------
-// body of the loop for capture_loop: iteration 0 (tallied), iteration 1 and
-// the decision, the update, the continue kernel
+// body of the loop for capture_loop: iteration 0 (tallied), iteration 1 with
+// the decision, the update
 LoopParts solve_parts(Solve &s) {
   LoopParts L;
   L.iter = [&s]() { return one_iteration(s, 0); };
   L.rest = [&s](cudaGraphConditionalHandle upd, cudaGraphConditionalHandle loop) {
-    TRY(one_iteration(s, 1));
-    k_cg_decide<<<1, 1, 0, s.ctx->stream>>>(s.st, upd, loop, 1);
-    return launched(s.ctx, "cg_decide");
+    Handles h;
+    h.upd = upd;
+    h.loop = loop;
+    h.in_graph = 1;
+    return one_iteration(s, 1, h);
   };
   L.update = [&s]() { return body_update(s); };
   return L;
@@ -908,7 +1022,7 @@ int cg_solve(hmc_ctx *ctx, const Geo &g, const hmc_gauge &Uh, const hmc_gauge *U
         pairs = whole_pairs < 1 ? 1 : whole_pairs;
       }
       const int k0 = h.iter;
-      for (int j = 0; !st && j < pairs; ++j) st = body_pair(s, 0, 0);
+      for (int j = 0; !st && j < pairs; ++j) st = body_pair(s);
       if (!st) st = read_state(s, &h);
       const double rr_now = h.rr[h.iter & 1];
       const int did = h.iter - k0;
