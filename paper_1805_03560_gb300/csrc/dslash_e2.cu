@@ -61,7 +61,8 @@ __global__ void __launch_bounds__(DS_NT, 3) k_dslash_e2(const DslashArgs a) {
         cp_async16(ls + q * DS_NT, lk + (q / 3) * lr + (q % 3) * lc);
     };
     AccE2 s;
-    zero_e2(s);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) s.up[q] = s.dn[q] = cdd2{{0ull, 0ull}, {0ull, 0ull}};
     fetch(0);
 #pragma unroll 1
     for (int k = 0; k < 8; ++k) {
@@ -75,7 +76,7 @@ __global__ void __launch_bounds__(DS_NT, 3) k_dslash_e2(const DslashArgs a) {
       hop_e2(
           p, [&] { if (k < 7) fetch(k + 1); },
           [&](int row, int q) { return ls[(3 * row + q) * DS_NT]; }, mu, fwd, fwd ? SF : -SF,
-          mu == 0 && c[0] == (fwd ? a.g.L[0] - 1 : 0), s);
+          mu == 0 && c[0] == (fwd ? a.g.L[0] - 1 : 0), false, s);
     }
     Cx<R> acc[12];
     unpack_e2(s, acc);

@@ -133,6 +133,30 @@ __device__ __forceinline__ void accumulate_rt(int mu, int S, Cx<R> acc[12], cons
   }
 }
 
+// acc = (w, -S B_mu^dag w): accumulate onto zero
+template <int MU, int S, typename R>
+__device__ __forceinline__ void spread(Cx<R> acc[12], const Cx<R> w[6]) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const Cx<R> w0 = w[a], w1 = w[3 + a];
+    acc[a] = w0;
+    acc[3 + a] = w1;
+    if (MU == 0) {
+      acc[6 + a] = S > 0 ? -w0 : w0;
+      acc[9 + a] = S > 0 ? -w1 : w1;
+    } else if (MU == 1) {
+      acc[6 + a] = S > 0 ? -ti(w1) : ti(w1);
+      acc[9 + a] = S > 0 ? -ti(w0) : ti(w0);
+    } else if (MU == 2) {
+      acc[6 + a] = S > 0 ? -w1 : w1;
+      acc[9 + a] = S > 0 ? w0 : -w0;
+    } else {
+      acc[6 + a] = S > 0 ? -ti(w0) : ti(w0);
+      acc[9 + a] = S > 0 ? ti(w1) : -ti(w1);
+    }
+  }
+}
+
 // project and accumulate of a direction known at run time (uniform over a warp)
 template <int S, typename R>
 __device__ __forceinline__ void project_mu(int mu, const Cx<R> p[12], Cx<R> h[6]) {
@@ -141,6 +165,15 @@ __device__ __forceinline__ void project_mu(int mu, const Cx<R> p[12], Cx<R> h[6]
     case 1: project<1, S>(p, h); break;
     case 2: project<2, S>(p, h); break;
     default: project<3, S>(p, h); break;
+  }
+}
+template <int S, typename R>
+__device__ __forceinline__ void spread_mu(int mu, Cx<R> acc[12], const Cx<R> w[6]) {
+  switch (mu) {
+    case 0: spread<0, S>(acc, w); break;
+    case 1: spread<1, S>(acc, w); break;
+    case 2: spread<2, S>(acc, w); break;
+    default: spread<3, S>(acc, w); break;
   }
 }
 template <int S, typename R>
@@ -188,10 +221,9 @@ __device__ __forceinline__ void project_e2(const float4 p[12], f32x2 S, f32x2 sg
 }
 
 template <int MU>
-__device__ __forceinline__ void accumulate_e2(AccE2 &acc, const cdd2 w[3], f32x2 S) {
+__device__ __forceinline__ void accumulate_e2(AccE2 &acc, const cdd2 w[3], f32x2 S, bool first) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    acc.up[a] = {add(acc.up[a].re, w[a].re), add(acc.up[a].im, w[a].im)};
     const cdd2 v = MU == 1 || MU == 2 ? cdd2{swap2(w[a].re), swap2(w[a].im)} : w[a];
     // -S v (mu 0), -S i v (1), (-S, S) v (2), (-S, S) i v (3)
     cdd2 t;
@@ -199,16 +231,22 @@ __device__ __forceinline__ void accumulate_e2(AccE2 &acc, const cdd2 w[3], f32x2
     if (MU == 1) t = {flip2(v.im, S), flip2(v.re, S ^ kNegBoth)};
     if (MU == 2) t = {flip2(v.re, S ^ kNeg0), flip2(v.im, S ^ kNeg0)};
     if (MU == 3) t = {flip2(v.im, S ^ kNeg1), flip2(v.re, S ^ kNeg0)};
-    acc.dn[a] = {add(acc.dn[a].re, t.re), add(acc.dn[a].im, t.im)};
+    if (first) {
+      acc.up[a] = w[a];
+      acc.dn[a] = t;
+    } else {
+      acc.up[a] = {add(acc.up[a].re, w[a].re), add(acc.up[a].im, w[a].im)};
+      acc.dn[a] = {add(acc.dn[a].re, t.re), add(acc.dn[a].im, t.im)};
+    }
   }
 }
 
 // p: the neighbour's spinor, dead once projected() is called; link(r, k): the
 // element U[r][k] of a forward hop's link, U[k][r] of a backward hop's; s: +1 or
-// -1 (the sign of gamma_mu), wrap: boundary sign
+// -1 (the sign of gamma_mu), wrap: boundary sign, first: acc is assigned
 template <typename Done, typename Link>
 __device__ __forceinline__ void hop_e2(const float4 p[12], Done projected, Link link, int mu,
-                                       bool fwd, int s, bool wrap, AccE2 &acc) {
+                                       bool fwd, int s, bool wrap, bool first, AccE2 &acc) {
   const f32x2 S = s > 0 ? 0ull : kNegBoth, sgn = wrap ? kNegBoth : 0ull;
   cdd2 h[3];
   switch (mu) {
@@ -233,17 +271,13 @@ __device__ __forceinline__ void hop_e2(const float4 p[12], Done projected, Link 
       w[r] = k == 0 ? cmul(ud, h[0], nh[0]) : cmac(w[r], ud, h[k], nh[k]);
     }
   switch (mu) {
-    case 0: accumulate_e2<0>(acc, w, S); break;
-    case 1: accumulate_e2<1>(acc, w, S); break;
-    case 2: accumulate_e2<2>(acc, w, S); break;
-    default: accumulate_e2<3>(acc, w, S); break;
+    case 0: accumulate_e2<0>(acc, w, S, first); break;
+    case 1: accumulate_e2<1>(acc, w, S, first); break;
+    case 2: accumulate_e2<2>(acc, w, S, first); break;
+    default: accumulate_e2<3>(acc, w, S, first); break;
   }
 }
 
-__device__ __forceinline__ void zero_e2(AccE2 &acc) {
-#pragma unroll
-  for (int a = 0; a < 3; ++a) acc.up[a] = acc.dn[a] = cdd2{{0ull, 0ull}, {0ull, 0ull}};
-}
 __device__ __forceinline__ void unpack_e2(const AccE2 &acc, Cx<df64> v[12]) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) {

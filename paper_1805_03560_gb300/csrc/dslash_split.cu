@@ -143,13 +143,14 @@ __global__ void __launch_bounds__(SPLIT_NT, split_min_blocks<SP>()) k_dslash_spl
   };
   double alpha_d = 0.0;
   Cx<R> acc[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = {R(0), R(0)};
   if constexpr (SP == HMC_F64E) {
     griddep_wait();
     if (a.gate && *a.gate == 0) return;
     AccE2 e2;
-    if constexpr (FMT == 18) zero_e2(e2);
+    if constexpr (FMT != 18) {
+#pragma unroll
+      for (int k = 0; k < 12; ++k) acc[k] = {R(0), R(0)};
+    }
 #pragma unroll 1
     for (int d = 0; d < 2; ++d) {
       const int S = d ? -SF : SF;
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(SPLIT_NT, split_min_blocks<SP>()) k_dslash_spl
         for (int k = 0; k < 12; ++k) p[k] = __ldg(in + (size_t)k * Vh);
         const size_t sr = (size_t)(d ? 1 : 3) * Vh, sc = (size_t)(d ? 3 : 1) * Vh;
         hop_e2(p, [] {}, [&](int r, int k) { return __ldg(lk + r * sr + k * sc); }, mu, d == 0,
-               S, d ? wb : wf, e2);
+               S, d ? wb : wf, d == 0, e2);
       } else {
         Cx<R> psi[12], u[9], hs[6], w[6];
         SIO::load(a.in, Vh, d ? hb : hf, psi);
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(SPLIT_NT, split_min_blocks<SP>()) k_dslash_spl
     project_mu<SF>(mu, pf, hs);
     flip(wf, hs);
     mul_link(uf, hs, w);
-    accumulate_mu<SF>(mu, acc, w);
+    spread_mu<SF>(mu, acc, w);
     project_mu<-SF>(mu, pb, hs);
     flip(wb, hs);
     mul_link_dag(ub, hs, w);
