@@ -164,12 +164,13 @@ int hmc_ctx_set_timing(hmc_ctx *ctx, int enable);
  * mapping) whose blocks first ask for a bulk L2 prefetch of the links they will
  * read (12-real FP32, F16 and BF16 links, one right-hand side; bit-identical
  * results; elsewhere variant 0 or 2 runs).  Default -1: for n_rhs > 1 in
- * FP32/FP16 the multi-right-hand-side kernel with 2 (else 3) per thread where
- * that divides n_rhs, otherwise paired loads for LINK18, for half storage and,
- * in FP32, where they fill the GPU better (by the lattice size).  With -1 and -2, one right-hand side in FP64,
- * FP32 or emulated FP64 on a lattice too small to fill the GPU runs one thread
- * per site and direction (the four directions' sums added last: within
- * rounding of the other variants).  -2: autotune: the first launch of each class
+ * F16/BF16 and in FP32 with LINK18 the multi-right-hand-side kernel with 2
+ * (else 3) per thread where that divides n_rhs, otherwise paired loads for
+ * LINK18, for half storage with one right-hand side and, in FP32, where they
+ * fill the GPU better (by the lattice size).  With -1 and -2, one right-hand
+ * side in FP64, FP32 or emulated FP64 on a lattice too small to fill the GPU
+ * runs one thread per site and direction (the four directions' sums added last:
+ * within rounding of the other variants).  -2: autotune: the first launch of each class
  * (precision, link format, dagger, n_rhs, lattice) that can be repeated without
  * changing its result times every applicable variant (one warm-up and three
  * timed launches each, synchronising the stream) and the class keeps the
@@ -179,8 +180,8 @@ int hmc_ctx_set_timing(hmc_ctx *ctx, int enable);
 /* HMC_OPT_CG_GRAPH: 1 (default) runs every CG solve of hmc_cg_solve and
  * hmc_cg_solve_multi (and every solve inside the force, action and trajectory
  * calls) as one CUDA graph captured per solve: a while node over the loop body
- * (two iterations, the second ending in the decision), the reliable update in an if node,
- * the convergence, reliable-update and iteration-limit decisions taken on the
+ * (two iterations, the second ending in the decision), the reliable update in
+ * an if node, the convergence, reliable-update and iteration-limit decisions taken on the
  * device (for a batched solve: for all systems together), the host reading the
  * solver state once at the end.  The graph runs on a stream of the library's
  * own that is ordered after the caller's stream and before its next work.

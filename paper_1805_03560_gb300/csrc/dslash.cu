@@ -559,13 +559,22 @@ static int mr_default(int sprec, int n_rhs) {
 // on, where the last one counts little, the paired form (32^3 x 64 564.0 /
 // 557.7).
 static int default_variant(const hmc_ctx *ctx, int fmt, int sprec, int n_rhs, int nb) {
+  // several right-hand sides: NR per thread where half storage makes the
+  // link's conversion and rebuilding the larger part (BF16 Mhat, 12 right-hand
+  // sides on 24^3 x 48, 2 per thread / 1: 505 / 575 us); in FP32 one per thread
+  // reads its spinors in whole lines (Mhat on 24^3 x 48, 2 / 4 / 8 / 12
+  // right-hand sides, 2 per thread 129 / 237 / 452 / 682 us, 1 per thread 110 /
+  // 200 / 376 / 553 us)
   const int nr = mr_default(sprec, n_rhs);
-  if (nr) return 2 + nr;
+  if (nr && (sprec != HMC_F32 || fmt == 18)) return 2 + nr;
   if (fmt == 18) return 2;
-  if (n_rhs > 1) return 0;
+  if (n_rhs > 1 && sprec != HMC_F32) return 0;
   if (sprec == HMC_F16 || sprec == HMC_BF16) return 2;
   if (sprec != HMC_F32) return 0;
   const int w4 = blocks_for(nb, 4 * ctx->sm_count), w6 = blocks_for(nb, 6 * ctx->sm_count);
+  // (several right-hand sides, paired / single: 2 on 16^3 x 32 23.1 / 25.5 us, 12 on
+  // 24^3 x 48 569 / 553: only for a clearly fuller last wave)
+  if (n_rhs > 1) return 16 * 4 * w4 < 15 * 6 * w6 ? 2 : 0;
   return w4 == 1 || w4 >= 8 || 4 * w4 < 6 * w6 ? 2 : 0;
 }
 
