@@ -6,6 +6,7 @@ Importing this module loads libhmc.so and raises if it is missing: there is no
 CPU fallback.
 """
 import ctypes
+import functools
 import os
 
 import numpy as np
@@ -163,6 +164,17 @@ def lib():
 
 def lattice(L):
     return Lat((ctypes.c_int * 4)(*[int(v) for v in L]))
+
+
+@functools.lru_cache(maxsize=64)
+def _lat_ref_of(L):
+    return ctypes.byref(lattice(L))
+
+
+def _lat_ref(L):
+    """The lattice argument of a call.  Built once per lattice: making the
+    ctypes structure took 4 of the 16 us of an Mhat call on 8^3 x 16."""
+    return _lat_ref_of(tuple(L))
 
 
 def _ref(x):
@@ -340,17 +352,17 @@ class Context:
     # ---- allocation ---------------------------------------------------------
     def new_spinor(self, L, prec, n_rhs=1):
         """Uninitialised half-spinor field of precision prec, n_rhs right-hand sides."""
-        n = lib().hmc_spinor_bytes(_ref(lattice(L)), prec, n_rhs)
+        n = lib().hmc_spinor_bytes(_lat_ref(L), prec, n_rhs)
         return Field(self._bytes(n), "spinor", prec, n_rhs)
 
     def new_gauge(self, L, prec, fmt):
         """Uninitialised gauge field of precision prec and link format fmt (LINK18 or LINK12)."""
-        n = lib().hmc_gauge_bytes(_ref(lattice(L)), prec, fmt)
+        n = lib().hmc_gauge_bytes(_lat_ref(L), prec, fmt)
         return Field(self._bytes(n), "gauge", prec, fmt=fmt)
 
     def new_algebra(self, L):
         """Zeroed algebra field (momenta or forces: 8 FP64 components per link)."""
-        n = lib().hmc_algebra_bytes(_ref(lattice(L)))
+        n = lib().hmc_algebra_bytes(_lat_ref(L))
         t = self.torch.zeros(int(n) // 8, dtype=self.torch.float64, device=f"cuda:{self.device}")
         return Field(t, "algebra", F64)
 
@@ -366,7 +378,7 @@ class Context:
         self._stream()
         Uc = self._canon(U)
         f = self.new_gauge(L, prec, fmt)
-        st = lib().hmc_pack_gauge(self.h, _ref(lattice(L)), _dp(Uc), f.ptr(), prec, fmt)
+        st = lib().hmc_pack_gauge(self.h, _lat_ref(L), _dp(Uc), f.ptr(), prec, fmt)
         self._check(st, "hmc_pack_gauge")
         return f
 
@@ -375,7 +387,7 @@ class Context:
         self._stream()
         V = int(np.prod(L))
         out = self.torch.empty((V, 4, 3, 3, 2), dtype=self.torch.float64, device=f"cuda:{self.device}")
-        st = lib().hmc_unpack_gauge(self.h, _ref(lattice(L)), f.ptr(), f.prec, f.fmt, _dp(out))
+        st = lib().hmc_unpack_gauge(self.h, _lat_ref(L), f.ptr(), f.prec, f.fmt, _dp(out))
         self._check(st, "hmc_unpack_gauge")
         return self.torch.view_as_complex(out)
 
@@ -385,7 +397,7 @@ class Context:
         c = self._canon(psi)
         n_rhs = 1 if c.dim() == 4 else c.shape[0]
         f = self.new_spinor(L, prec, n_rhs)
-        st = lib().hmc_pack_spinor(self.h, _ref(lattice(L)), _dp(c), f.ptr(), prec, n_rhs)
+        st = lib().hmc_pack_spinor(self.h, _lat_ref(L), _dp(c), f.ptr(), prec, n_rhs)
         self._check(st, "hmc_pack_spinor")
         return f
 
@@ -395,7 +407,7 @@ class Context:
         Vh = int(np.prod(L)) // 2
         shape = (Vh, 4, 3, 2) if f.n_rhs == 1 else (f.n_rhs, Vh, 4, 3, 2)
         out = self.torch.empty(shape, dtype=self.torch.float64, device=f"cuda:{self.device}")
-        st = lib().hmc_unpack_spinor(self.h, _ref(lattice(L)), f.ptr(), f.prec, f.n_rhs, _dp(out))
+        st = lib().hmc_unpack_spinor(self.h, _lat_ref(L), f.ptr(), f.prec, f.n_rhs, _dp(out))
         self._check(st, "hmc_unpack_spinor")
         return self.torch.view_as_complex(out)
 
@@ -404,7 +416,7 @@ class Context:
         self._stream()
         c = self._canon(A)
         f = self.new_algebra(L)
-        st = lib().hmc_pack_algebra(self.h, _ref(lattice(L)), _dp(c), _dp(f.data))
+        st = lib().hmc_pack_algebra(self.h, _lat_ref(L), _dp(c), _dp(f.data))
         self._check(st, "hmc_pack_algebra")
         return f
 
@@ -413,7 +425,7 @@ class Context:
         self._stream()
         V = int(np.prod(L))
         out = self.torch.empty((V, 4, 8), dtype=self.torch.float64, device=f"cuda:{self.device}")
-        st = lib().hmc_unpack_algebra(self.h, _ref(lattice(L)), _dp(f.data), _dp(out))
+        st = lib().hmc_unpack_algebra(self.h, _lat_ref(L), _dp(f.data), _dp(out))
         self._check(st, "hmc_unpack_algebra")
         return out
 
@@ -422,7 +434,7 @@ class Context:
         """out (parity out_parity) = H_{p,1-p} inp, or gamma_5 H gamma_5 with dagger."""
         self._stream()
         g = U.gauge()
-        st = lib().hmc_dslash(self.h, _ref(lattice(L)), ctypes.byref(g), out.ptr(), inp.ptr(),
+        st = lib().hmc_dslash(self.h, _lat_ref(L), ctypes.byref(g), out.ptr(), inp.ptr(),
                               out_parity, int(dagger), inp.prec, inp.n_rhs)
         self._check(st, "hmc_dslash")
         return out
@@ -435,7 +447,7 @@ class Context:
         ks = None
         if kappas is not None:
             ks = np.ascontiguousarray(kappas, dtype=np.float64)
-        st = lib().hmc_mhat(self.h, _ref(lattice(L)), ctypes.byref(g), out.ptr(), inp.ptr(), kappa,
+        st = lib().hmc_mhat(self.h, _lat_ref(L), ctypes.byref(g), out.ptr(), inp.ptr(), kappa,
                             int(dagger), inp.prec, inp.n_rhs,
                             ks.ctypes.data_as(_P) if ks is not None else None)
         self._check(st, "hmc_mhat")
@@ -450,7 +462,7 @@ class Context:
         gl = U_lo.gauge() if U_lo is not None else None
         opts = SolverOpts(F64, 0.1, 16, F64, f64_emul, SOLVER_BICGSTAB)
         stats = SolveStats()
-        st = lib().hmc_bicgstab_solve(self.h, _ref(lattice(L)), ctypes.byref(gh),
+        st = lib().hmc_bicgstab_solve(self.h, _lat_ref(L), ctypes.byref(gh),
                                       ctypes.byref(gl) if gl is not None else None, x.ptr(),
                                       b.ptr(), kappa, int(bool(dagger)), tol, max_iter,
                                       ctypes.byref(opts), ctypes.byref(stats))
@@ -467,7 +479,7 @@ class Context:
         gl = U_lo.gauge() if U_lo is not None else None
         opts = SolverOpts(inner_prec, reliable_delta, check_every, F64, f64_emul)
         stats = SolveStats()
-        st = lib().hmc_cg_solve(self.h, _ref(lattice(L)), ctypes.byref(gh),
+        st = lib().hmc_cg_solve(self.h, _lat_ref(L), ctypes.byref(gh),
                                 ctypes.byref(gl) if gl is not None else None, x.ptr(), phi.ptr(),
                                 kappa, tol, max_iter, ctypes.byref(opts), ctypes.byref(stats))
         res = {"iterations": stats.iterations, "reliable_updates": stats.reliable_updates,
@@ -487,7 +499,7 @@ class Context:
         assert len(ks) == n
         opts = SolverOpts(inner_prec, reliable_delta, check_every, F64, f64_emul)
         stats = (SolveStats * n)()
-        st = lib().hmc_cg_solve_multi(self.h, _ref(lattice(L)), ctypes.byref(gh),
+        st = lib().hmc_cg_solve_multi(self.h, _lat_ref(L), ctypes.byref(gh),
                                       ctypes.byref(gl) if gl is not None else None, x.ptr(),
                                       phi.ptr(), ks.ctypes.data_as(_P), n, tol, max_iter,
                                       ctypes.byref(opts), stats)
@@ -515,7 +527,7 @@ class Context:
         flt, keep = self._filter(b, alpha)
         opts = SolverOpts(inner_prec, reliable_delta, 16, force_prec, f64_emul, solver)
         stats = SolveStats()
-        st = lib().hmc_force_pf(self.h, _ref(lattice(L)), ctypes.byref(gh),
+        st = lib().hmc_force_pf(self.h, _lat_ref(L), ctypes.byref(gh),
                                 ctypes.byref(gl) if gl is not None else None, phi.ptr(), kappa,
                                 ctypes.byref(flt) if flt is not None else None, coeff,
                                 _dp(F.data), tol, ctypes.byref(opts), ctypes.byref(stats))
@@ -532,7 +544,7 @@ class Context:
         flt, keep = self._filter(b, alpha)
         opts = SolverOpts(inner_prec, reliable_delta, 16, force_prec, f64_emul, solver)
         stats = SolveStats()
-        st = lib().hmc_force_fratio(self.h, _ref(lattice(L)), ctypes.byref(gh),
+        st = lib().hmc_force_fratio(self.h, _lat_ref(L), ctypes.byref(gh),
                                     ctypes.byref(gl) if gl is not None else None, phi.ptr(),
                                     kappa, ctypes.byref(flt), kappa_a, coeff, _dp(F.data), tol,
                                     ctypes.byref(opts), ctypes.byref(stats))
@@ -548,7 +560,7 @@ class Context:
         flt, keep = self._filter(b, alpha)
         opts = SolverOpts(inner_prec, 0.1, 16, F64, f64_emul, solver)
         out = ctypes.c_double(0)
-        st = lib().hmc_action_fratio(self.h, _ref(lattice(L)), ctypes.byref(gh),
+        st = lib().hmc_action_fratio(self.h, _lat_ref(L), ctypes.byref(gh),
                                      ctypes.byref(gl) if gl is not None else None, phi.ptr(),
                                      kappa, ctypes.byref(flt), kappa_a, tol, ctypes.byref(opts),
                                      ctypes.byref(out), None)
@@ -565,7 +577,7 @@ class Context:
         flt, keep = self._filter(b, alpha)
         opts = SolverOpts(inner_prec, 0.1, 16, F64, f64_emul, solver)
         out = ctypes.c_double(0)
-        st = lib().hmc_action_pf(self.h, _ref(lattice(L)), ctypes.byref(gh),
+        st = lib().hmc_action_pf(self.h, _lat_ref(L), ctypes.byref(gh),
                                  ctypes.byref(gl) if gl is not None else None, phi.ptr(), kappa,
                                  ctypes.byref(flt) if flt is not None else None, tol,
                                  ctypes.byref(opts), ctypes.byref(out), None)
@@ -578,7 +590,7 @@ class Context:
         self._stream()
         g = U.gauge()
         act = ctypes.c_double(0)
-        st = lib().hmc_force_hopexp(self.h, _ref(lattice(L)), ctypes.byref(g), beta, kappa, k,
+        st = lib().hmc_force_hopexp(self.h, _lat_ref(L), ctypes.byref(g), beta, kappa, k,
                                     coeff, _dp(F.data) if F is not None else None,
                                     ctypes.byref(act) if want_action else None)
         self._check(st, "hmc_force_hopexp")
@@ -589,7 +601,7 @@ class Context:
         self._stream()
         g = U.gauge()
         out = ctypes.c_double(0)
-        st = lib().hmc_plaquette(self.h, _ref(lattice(L)), ctypes.byref(g), ctypes.byref(out))
+        st = lib().hmc_plaquette(self.h, _lat_ref(L), ctypes.byref(g), ctypes.byref(out))
         self._check(st, "hmc_plaquette")
         return out.value
 
@@ -615,7 +627,7 @@ class Context:
         gl = U_lo.gauge() if U_lo is not None else None
         opts = SolverOpts(F64, 0.1, 16, F64, f64_emul)
         stats = SolveStats()
-        st = lib().hmc_poly_solve(self.h, _ref(lattice(L)), ctypes.byref(gh),
+        st = lib().hmc_poly_solve(self.h, _lat_ref(L), ctypes.byref(gh),
                                   ctypes.byref(gl) if gl is not None else None, x.ptr(), b.ptr(),
                                   c.ctypes.data_as(_P), len(c) - 1, kappa, tol, max_iter,
                                   ctypes.byref(opts), ctypes.byref(stats))
@@ -633,7 +645,7 @@ class Context:
     def pack_spinors(self, L, fields):
         """n F64 even fields stored one after another (not interleaved), the
         layout of the pseudo-fermion fields of a mass-preconditioned chain."""
-        nb = int(lib().hmc_spinor_bytes(_ref(lattice(L)), F64, 1))
+        nb = int(lib().hmc_spinor_bytes(_lat_ref(L), F64, 1))
         out = Field(self._bytes(nb * len(fields)), "spinor", F64, 1)
         out.n_fields = len(fields)
         for j, f in enumerate(fields):
@@ -643,7 +655,7 @@ class Context:
 
     def unpack_spinors(self, L, f):
         """The consecutive F64 fields of pack_spinors, stacked as complex128 [n, Vh, 4, 3]."""
-        nb = int(lib().hmc_spinor_bytes(_ref(lattice(L)), F64, 1))
+        nb = int(lib().hmc_spinor_bytes(_lat_ref(L), F64, 1))
         res = []
         for j in range(f.data.numel() // nb):
             one = Field(f.data[j * nb:(j + 1) * nb], "spinor", F64, 1)
@@ -666,7 +678,7 @@ class Context:
         gl = U_lo.gauge() if U_lo is not None else None
         opts = SolverOpts(inner_prec, reliable_delta, 16, force_prec, f64_emul)
         stats = SolveStats()
-        st = lib().hmc_force_mp(self.h, _ref(lattice(L)), ctypes.byref(gh),
+        st = lib().hmc_force_mp(self.h, _lat_ref(L), ctypes.byref(gh),
                                 ctypes.byref(gl) if gl is not None else None, phis.ptr(), n, ka,
                                 kb, coeff, _dp(F.data), tol, ctypes.byref(opts),
                                 ctypes.byref(stats))
@@ -683,7 +695,7 @@ class Context:
         gl = U_lo.gauge() if U_lo is not None else None
         opts = SolverOpts(inner_prec, 0.1, 16, F64, f64_emul)
         out = ctypes.c_double(0)
-        st = lib().hmc_action_mp(self.h, _ref(lattice(L)), ctypes.byref(gh),
+        st = lib().hmc_action_mp(self.h, _lat_ref(L), ctypes.byref(gh),
                                  ctypes.byref(gl) if gl is not None else None, phis.ptr(), n, ka,
                                  kb, tol, ctypes.byref(opts), ctypes.byref(out), None)
         self._check(st, "hmc_action_mp")
@@ -700,7 +712,7 @@ class Context:
         gl = U_lo.gauge() if U_lo is not None else None
         opts = SolverOpts(inner_prec, 0.1, 16, F64, f64_emul)
         out = Field(self._bytes(etas.data.numel()), "spinor", F64, 1)
-        st = lib().hmc_heatbath_mp(self.h, _ref(lattice(L)), ctypes.byref(gh),
+        st = lib().hmc_heatbath_mp(self.h, _lat_ref(L), ctypes.byref(gh),
                                    ctypes.byref(gl) if gl is not None else None, etas.ptr(), n,
                                    ka, kb, tol, ctypes.byref(opts), out.ptr(), None)
         self._check(st, "hmc_heatbath_mp")
@@ -714,7 +726,7 @@ class Context:
         V = int(np.prod(L))
         out = self.torch.empty((V, 4, 3, 3, 2), dtype=self.torch.float64,
                                device=f"cuda:{self.device}")
-        st = lib().hmc_link_gradient(self.h, _ref(lattice(L)), _dp(c), _dp(F.data), float(scale),
+        st = lib().hmc_link_gradient(self.h, _lat_ref(L), _dp(c), _dp(F.data), float(scale),
                                      _dp(out))
         self._check(st, "hmc_link_gradient")
         return self.torch.view_as_complex(out)
@@ -725,7 +737,7 @@ class Context:
         self._stream()
         g = U.gauge()
         c = np.ascontiguousarray(coeffs, dtype=np.float64)
-        st = lib().hmc_poly_apply(self.h, _ref(lattice(L)), ctypes.byref(g), out.ptr(), inp.ptr(),
+        st = lib().hmc_poly_apply(self.h, _lat_ref(L), ctypes.byref(g), out.ptr(), inp.ptr(),
                                   c.ctypes.data_as(_P), len(c) - 1, kappa, inp.prec,
                                   _dp(horner_store) if horner_store is not None else None)
         self._check(st, "hmc_poly_apply")
@@ -734,20 +746,20 @@ class Context:
     def update_links(self, L, U, P, eps):
         """U <- exp(eps Pi) U with Pi from the algebra field P, reunitarised (native FP64)."""
         self._stream()
-        st = lib().hmc_update_links(self.h, _ref(lattice(L)), U.ptr(), _dp(P.data), eps)
+        st = lib().hmc_update_links(self.h, _lat_ref(L), U.ptr(), _dp(P.data), eps)
         self._check(st, "hmc_update_links")
 
     def update_momenta(self, L, P, F, eps):
         """P <- P - eps F."""
         self._stream()
-        st = lib().hmc_update_momenta(self.h, _ref(lattice(L)), _dp(P.data), _dp(F.data), eps)
+        st = lib().hmc_update_momenta(self.h, _lat_ref(L), _dp(P.data), _dp(F.data), eps)
         self._check(st, "hmc_update_momenta")
 
     def kinetic(self, L, P):
         """Kinetic term (1/2)(Pi, Pi) = (1/2) sum_a P_a^2 of an algebra field."""
         self._stream()
         out = ctypes.c_double(0)
-        st = lib().hmc_kinetic(self.h, _ref(lattice(L)), _dp(P.data), ctypes.byref(out))
+        st = lib().hmc_kinetic(self.h, _lat_ref(L), _dp(P.data), ctypes.byref(out))
         self._check(st, "hmc_kinetic")
         return out.value
 
@@ -772,7 +784,7 @@ class Context:
             measure_forces=measure_forces, solver=solver, level_steps=level_steps,
             term_level=term_level)
         res = TrajResult()
-        st = lib().hmc_trajectory(self.h, _ref(lattice(L)), U.ptr(), ctypes.byref(prm),
+        st = lib().hmc_trajectory(self.h, _lat_ref(L), U.ptr(), ctypes.byref(prm),
                                   _dp(P.data), eta.ptr(), u, ctypes.byref(res),
                                   U_end.ptr() if U_end is not None else None,
                                   _dp(P_end.data) if P_end is not None else None)
@@ -821,17 +833,17 @@ class Context:
         """Momenta with N(0,1) components from (seed, counter) (hmc_random_momenta)."""
         self._stream()
         P = P if P is not None else self.new_algebra(L)
-        st = lib().hmc_random_momenta(self.h, _ref(lattice(L)), _dp(P.data), seed, counter)
+        st = lib().hmc_random_momenta(self.h, _lat_ref(L), _dp(P.data), seed, counter)
         self._check(st, "hmc_random_momenta")
         return P
 
     def random_sources(self, L, n, seed, counter):
         """n consecutive F64 even sources, density exp(-|eta|^2) (hmc_random_sources)."""
         self._stream()
-        nb = int(lib().hmc_spinor_bytes(_ref(lattice(L)), F64, 1))
+        nb = int(lib().hmc_spinor_bytes(_lat_ref(L), F64, 1))
         out = Field(self._bytes(nb * n), "spinor", F64, 1)
         out.n_fields = n
-        st = lib().hmc_random_sources(self.h, _ref(lattice(L)), out.ptr(), n, seed, counter)
+        st = lib().hmc_random_sources(self.h, _lat_ref(L), out.ptr(), n, seed, counter)
         self._check(st, "hmc_random_sources")
         return out
 
@@ -852,7 +864,7 @@ class Context:
         prm = self._traj_params(keep, **traj)
         cp = ChainParams(seed, counter0, n_traj, spike_threshold)
         res = (TrajResult * max(n_traj, 1))()
-        st = lib().hmc_chain(self.h, _ref(lattice(L)), U.ptr(), ctypes.byref(prm),
+        st = lib().hmc_chain(self.h, _lat_ref(L), U.ptr(), ctypes.byref(prm),
                              ctypes.byref(cp), res)
         self._check(st, "hmc_chain")
         return [{f: getattr(res[t], f) for f, _ in TrajResult._fields_} for t in range(n_traj)]
@@ -904,7 +916,7 @@ class Context:
         if c is not None:
             ac = np.ascontiguousarray(c, dtype=np.float64); keep.append(ac); prm.c = ac.ctypes.data
         res = TrajResult()
-        st = lib().hmc_md_evolve(self.h, _ref(lattice(L)), U.ptr(), _dp(P.data), phi.ptr(),
+        st = lib().hmc_md_evolve(self.h, _lat_ref(L), U.ptr(), _dp(P.data), phi.ptr(),
                                  ctypes.byref(prm), ctypes.byref(res))
         self._check(st, "hmc_md_evolve")
         return {f: getattr(res, f) for f, _ in TrajResult._fields_ if f not in
