@@ -723,7 +723,7 @@ int dslash(hmc_ctx *ctx, const DslashArgs &a, const hmc_gauge &U, int sprec, int
   if (split) {
     if (nblocks) *nblocks = dslash_split_blocks(a.g);
     TimedLaunch timer(ctx, cls, bytes);
-    if (!launch_dslash_split(la, sprec, U.fmt, dagger, st))
+    if (!launch_dslash_split(ctx, la, sprec, U.fmt, dagger))
       return fail(ctx, HMC_EINVAL, "dslash: unsupported precision %d / link format %d", sprec,
                   U.fmt);
     return launched(ctx, cls);
