@@ -244,6 +244,8 @@ int dslash(hmc_ctx *ctx, const DslashArgs &a, const hmc_gauge &U, int sprec, int
 int dslash_tune(hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, int sprec, int n_rhs, void *out,
                 const void *in);
 
+// n complex numbers of 16 bytes, F64 -> F64E
+void chunks_to_f64e(hmc_ctx *ctx, void *dst, const void *src, long long n);
 int zero_field(hmc_ctx *ctx, int prec, void *d, int S);
 int copy_convert(hmc_ctx *ctx, int pd, int ps, void *d, const void *s, int S);
 int norm_partials(hmc_ctx *ctx, int prec, const void *v, int S, double *partials, int *nb);
@@ -260,6 +262,12 @@ int hop_force_multi(hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, int n, const
                     const void *const V[][2], double *F, double c, int sprec);
 int gauge_force(hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, double beta, double kappa, int k,
                 double coeff, double *F);
+// Kernels that use more dynamic shared memory than the default limit: raise
+// it on the current device (once per context, when it is created, so that no
+// launch does it while a stream is captured)
+cudaError_t dslash_e2_smem();
+cudaError_t hop_force_smem();
+cudaError_t gauge_force_smem();
 int gauge_action_sums(hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, int with_lines,
                       double *partials, double *dst);
 int gauge_action_coeffs(hmc_ctx *ctx, const Geo &g, double beta, double kappa, int k,

@@ -113,6 +113,32 @@ struct df64 {
   __device__ explicit operator float() const { return __fadd_rn(hi, lo); }
 };
 
+// df64(d) by integer operations on the bits where d lies well inside the float
+// range (else by the conversions): the FP64 pipe (two lanes per cycle and SM)
+// needs four passes for it.  The values are the same: hi = d rounded to
+// nearest even, lo = the exact remainder rounded.
+__device__ __forceinline__ df64 split_double(double d) {
+  const unsigned b1 = (unsigned)__double2hiint(d), b0 = (unsigned)__double2loint(d);
+  const unsigned e = (b1 >> 20) & 0x7ffu, s = b1 & 0x80000000u;
+  if (e - 960u >= 190u) return df64(d);
+  // 53-bit significand: its top 24 bits in h, the other 29 in rem
+  unsigned h = (((b1 & 0xfffffu) | 0x100000u) << 3) | (b0 >> 29);
+  const unsigned rem = b0 & 0x1fffffffu, inc = rem + (h & 1u) > 0x10000000u ? 1u : 0u;
+  h += inc;
+  return {__uint_as_float(s | (((e - 897u) << 23) + h)),
+          __fmul_rn(__int2float_rn((int)rem - (int)(inc << 29)),
+                    __uint_as_float(s | ((e - 948u) << 23)))};
+}
+
+// one complex number of 16 bytes, F64 <-> F64E
+__device__ __forceinline__ float4 to_f64e(double2 v) {
+  const df64 re = split_double(v.x), im = split_double(v.y);
+  return make_float4(re.hi, re.lo, im.hi, im.lo);
+}
+__device__ __forceinline__ double2 to_f64(float4 v) {
+  return make_double2((double)df64(v.x, v.y), (double)df64(v.z, v.w));
+}
+
 __device__ __forceinline__ df64 dd_two_sum(float a, float b) {
   const float s = __fadd_rn(a, b);
   const float bb = __fsub_rn(s, a);

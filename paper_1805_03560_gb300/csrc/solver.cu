@@ -105,6 +105,37 @@ __global__ void __launch_bounds__(BL_NT) k_copy(void *dst, const void *src, int 
   store_as<PD>(dst, S, i, a);
 }
 
+// F64 <-> F64E and copies of either: both hold one complex number per 16 bytes
+// in the same order, spinors and links alike, so these go over n 16-byte chunks,
+// one per thread and pass.  Memory bounds them; one site or link per thread
+// (twelve or nine strided loads, then the conversions on the FP64 pipe, then the
+// stores) ran at a third of its rate.  Measured on 24^3 x 48, that form -> this:
+// links to F64E 348 -> 175 us, the spinor conversions and copies of a filtered force
+// 53 -> 38 us on average, a kappa^4 trajectory on 12^3 x 24 43.3 -> 41.1 ms.
+enum ChunkOp { CHUNK_COPY, CHUNK_TO_F64E, CHUNK_TO_F64 };
+template <int OP>
+__global__ void __launch_bounds__(BL_NT) k_convert_chunks(void *dst, const void *src, long long n) {
+  const long long stride = (long long)gridDim.x * BL_NT;
+  for (long long i = (long long)blockIdx.x * BL_NT + threadIdx.x; i < n; i += stride) {
+    if (OP == CHUNK_COPY)
+      ((float4 *)dst)[i] = ((const float4 *)src)[i];
+    else if (OP == CHUNK_TO_F64E)
+      ((float4 *)dst)[i] = to_f64e(((const double2 *)src)[i]);
+    else
+      ((double2 *)dst)[i] = to_f64(((const float4 *)src)[i]);
+  }
+}
+
+template <int OP>
+static void chunks_l(hmc_ctx *ctx, void *dst, const void *src, long long n) {
+  const int nb = blocks_for(n, BL_NT), most = 32 * ctx->sm_count;
+  k_convert_chunks<OP><<<nb < most ? nb : most, BL_NT, 0, ctx->stream>>>(dst, src, n);
+}
+
+void chunks_to_f64e(hmc_ctx *ctx, void *dst, const void *src, long long n) {
+  chunks_l<CHUNK_TO_F64E>(ctx, dst, src, n);
+}
+
 template <int P>
 __global__ void __launch_bounds__(BL_NT) k_zero(void *dst, int S) {
   int i = blockIdx.x * BL_NT + threadIdx.x;
@@ -249,7 +280,7 @@ __global__ void __launch_bounds__(XP_NT, XP_BLOCKS) k_cg_xpay_chunks(
   // went the other way and left its last elements in L2)
   const auto at = [&](long long j) { return rev ? n - 1 - j : j; };
   const auto valid = [&](long long c) {
-    if (PL == HMC_F32) return (c / 192) * 32 + (c & 31) < S;
+    if (PL == HMC_F32) return !kBlockedF32 || (c / 192) * 32 + (c & 31) < S;
     return c < (long long)S * 12;
   };
   long long j = (long long)blockIdx.x * XP_NT + threadIdx.x;
@@ -510,7 +541,6 @@ static void copy_l(hmc_ctx *ctx, void *d, const void *s, int S) {
 
 int copy_convert(hmc_ctx *ctx, int pd, int ps, void *d, const void *s, int S) {
   switch (pd * 10 + ps) {
-    case HMC_F64 * 10 + HMC_F64: copy_l<HMC_F64, HMC_F64>(ctx, d, s, S); break;
     case HMC_F32 * 10 + HMC_F64: copy_l<HMC_F32, HMC_F64>(ctx, d, s, S); break;
     case HMC_F16 * 10 + HMC_F64: copy_l<HMC_F16, HMC_F64>(ctx, d, s, S); break;
     case HMC_F64 * 10 + HMC_F32: copy_l<HMC_F64, HMC_F32>(ctx, d, s, S); break;
@@ -520,9 +550,10 @@ int copy_convert(hmc_ctx *ctx, int pd, int ps, void *d, const void *s, int S) {
     case HMC_BF16 * 10 + HMC_F64: copy_l<HMC_BF16, HMC_F64>(ctx, d, s, S); break;
     case HMC_F64 * 10 + HMC_BF16: copy_l<HMC_F64, HMC_BF16>(ctx, d, s, S); break;
     case HMC_BF16 * 10 + HMC_BF16: copy_l<HMC_BF16, HMC_BF16>(ctx, d, s, S); break;
-    case HMC_F64E * 10 + HMC_F64: copy_l<HMC_F64E, HMC_F64>(ctx, d, s, S); break;
-    case HMC_F64 * 10 + HMC_F64E: copy_l<HMC_F64, HMC_F64E>(ctx, d, s, S); break;
-    case HMC_F64E * 10 + HMC_F64E: copy_l<HMC_F64E, HMC_F64E>(ctx, d, s, S); break;
+    case HMC_F64E * 10 + HMC_F64: chunks_l<CHUNK_TO_F64E>(ctx, d, s, 12LL * S); break;
+    case HMC_F64 * 10 + HMC_F64E: chunks_l<CHUNK_TO_F64>(ctx, d, s, 12LL * S); break;
+    case HMC_F64E * 10 + HMC_F64E:
+    case HMC_F64 * 10 + HMC_F64: chunks_l<CHUNK_COPY>(ctx, d, s, 12LL * S); break;
     default: return fail(ctx, HMC_EINVAL, "copy: unsupported precisions %d <- %d", pd, ps);
   }
   return launched(ctx, "copy");

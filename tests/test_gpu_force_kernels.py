@@ -64,3 +64,16 @@ def test_gauge_force(ctx, H, L, fmt):
     want = res[H.F64]
     assert np.abs(res[H.F64E] - want).max() <= 2e-13 * np.abs(want).max()
     assert np.abs(res[H.F32] - want).max() <= 2e-5 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("L", [(2, 2, 2, 2), (4, 6, 10, 14)])
+def test_force_with_exact_zeros(ctx, H, L):
+    """Links with zero entries and a source with zero components (values the
+    bitwise F64 -> F64E conversion leaves to the FP64 conversions)."""
+    U = ctx.pack_gauge(L, I.integer_links(L), 0, 18)
+    phi = I.gaussian_half(L, 2)
+    phi[::2, 1] = 0.0
+    phi = ctx.pack_spinor(L, phi, 0)
+    want = _force(ctx, H, L, U, phi, H.F64, 3)
+    got = _force(ctx, H, L, U, phi, H.F64E, 3)
+    assert np.abs(got - want).max() <= 2e-13 * np.abs(want).max()
