@@ -264,6 +264,9 @@ int hmc_ctx_create(int device, hmc_ctx **out) {
   if (!out) return HMC_EINVAL;
   *out = nullptr;
   if (cudaSetDevice(device) != cudaSuccess) return HMC_ECUDA;
+  if (dslash_e2_smem() != cudaSuccess || hop_force_smem() != cudaSuccess ||
+      gauge_force_smem() != cudaSuccess)
+    return HMC_ECUDA;
   hmc_ctx *c = new hmc_ctx();
   c->device = device;
   if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||

@@ -116,11 +116,16 @@ __global__ void __launch_bounds__(DS_NT, 3) k_dslash_e2(const DslashArgs a) {
 
 }  // namespace
 
+cudaError_t dslash_e2_smem() {
+  const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  const cudaError_t e = cudaFuncSetAttribute(k_dslash_e2<false>, at, E2_SMEM);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(k_dslash_e2<true>, at, E2_SMEM);
+}
+
 void launch_dslash_e2(DslashArgs a, int dagger, cudaStream_t st) {
   const int nb = blocks_for((long long)a.g.Vh * a.n_rhs, DS_NT);
   if (a.rev) a.rev = nb;
   const auto kernel = dagger ? k_dslash_e2<true> : k_dslash_e2<false>;
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, E2_SMEM);
   launch_pdl_smem(kernel, nb, DS_NT, E2_SMEM, st, a.pdl != 0, a);
 }
 

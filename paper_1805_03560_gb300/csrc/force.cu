@@ -226,8 +226,13 @@ __global__ void __launch_bounds__(HF_NT, 3) k_hop_force_e2(const HopForceArgs a)
 
 template <int FMT>
 static void launch_hop_force_e2(const HopForceArgs &a, int nb, cudaStream_t st) {
-  cudaFuncSetAttribute(k_hop_force_e2<FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, HF_SMEM);
   k_hop_force_e2<FMT><<<nb, HF_NT, HF_SMEM, st>>>(a);
+}
+
+cudaError_t hop_force_smem() {
+  const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  const cudaError_t e = cudaFuncSetAttribute(k_hop_force_e2<18>, at, HF_SMEM);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(k_hop_force_e2<12>, at, HF_SMEM);
 }
 
 int hop_force(hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, const void *We, const void *Wo,

@@ -351,6 +351,11 @@ static int hopexp_coeffs(hmc_ctx *ctx, const Geo &g, double beta, double kappa, 
   return HMC_OK;
 }
 
+cudaError_t gauge_force_smem() {
+  return cudaFuncSetAttribute(k_gauge_force_e2, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              GF_SMEM);
+}
+
 int gauge_force(hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, double beta, double kappa, int k,
                 double coeff, double *F) {
   double beff = beta, cl[4] = {0.0, 0.0, 0.0, 0.0};
@@ -374,7 +379,6 @@ int gauge_force(hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, double beta, dou
     case HMC_F32 * 100 + 12: k_gauge_force<HMC_F32, 12><<<nb, 128, 0, strm>>>(a); break;
     // emulated FP64: staples and U A in double-float, F accumulated in FP64
     case HMC_F64E * 100 + 18:
-      cudaFuncSetAttribute(k_gauge_force_e2, cudaFuncAttributeMaxDynamicSharedMemorySize, GF_SMEM);
       k_gauge_force_e2<<<8 * blocks_for(g.Vh, GF_NT), GF_NT, GF_SMEM, strm>>>(a);
       break;
     case HMC_F64E * 100 + 12: k_gauge_force<HMC_F64E, 12><<<nb, 128, 0, strm>>>(a); break;
