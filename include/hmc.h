@@ -170,8 +170,8 @@ int hmc_ctx_set_timing(hmc_ctx *ctx, int enable);
  * fill the GPU better (by the lattice size).  With -1 and -2, one right-hand
  * side in FP64, FP32 or emulated FP64 on a lattice too small to fill the GPU
  * runs one thread per site and direction (the four directions' sums added last:
- * within rounding of the other variants).  -2: autotune: the first launch of each class
- * (precision, link format, dagger, n_rhs, lattice) that can be repeated without
+ * within rounding of the other variants).  -2: autotune: the first launch of
+ * each class (precision, link format, dagger, n_rhs, lattice) that can be repeated without
  * changing its result times every applicable variant (one warm-up and three
  * timed launches each, synchronising the stream) and the class keeps the
  * fastest; the solvers tune their classes on scratch fields before iterating.
@@ -181,8 +181,8 @@ int hmc_ctx_set_timing(hmc_ctx *ctx, int enable);
  * hmc_cg_solve_multi (and every solve inside the force, action and trajectory
  * calls) as one CUDA graph captured per solve: a while node over the loop body
  * (two iterations, the second ending in the decision), the reliable update in
- * an if node, the convergence, reliable-update and iteration-limit decisions taken on the
- * device (for a batched solve: for all systems together), the host reading the
+ * an if node, the convergence, reliable-update and iteration-limit decisions
+ * taken on the device (for a batched solve: for all systems together), the host reading the
  * solver state once at the end.  The graph runs on a stream of the library's
  * own that is ordered after the caller's stream and before its next work.
  * BiCGstab passes replay one captured iteration in batches of 16, reading the
@@ -195,8 +195,10 @@ int hmc_ctx_set_timing(hmc_ctx *ctx, int enable);
  * xpay as programmatic dependent launches: each may be scheduled while the
  * kernel before it on the stream finishes its last blocks, and waits for that
  * kernel's completion (griddepcontrol.wait) before touching its data, so the
- * gap between dependent launches closes; results are bit-identical.  0
- * launches them normally. */
+ * gap between dependent launches closes; results are bit-identical.  (Native
+ * FP64 on lattices whose blocks spread evenly over the SMs in one wave is
+ * launched normally: blocks placed early share an SM's FP64 pipe.)  0 launches
+ * all of them normally. */
 #define HMC_OPT_PDL 4
 /* HMC_OPT_BATCH: how hmc_cg_solve_multi (and the batched solves of the
  * mass-preconditioned terms) run n_rhs > 1 systems: 1 in lock step (each
