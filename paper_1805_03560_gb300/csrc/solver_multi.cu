@@ -254,7 +254,7 @@ __global__ void k_mcontrol_init(MState *st, int n, double delta2, int max_iter, 
 // |r_q|^2 below its tolerance or delta^2 times its largest value since the
 // last update; plain: every live system converged on its recursive residual),
 // or the iteration limit; in a graph `upd` receives whether the update runs
-// and `loop` whether the loop goes on (as in k_cg_decide)
+// and `loop` whether the loop goes on (as in cg_decide)
 __global__ void k_mdecide(MState *st, cudaGraphConditionalHandle upd,
                           cudaGraphConditionalHandle loop, int in_graph) {
   int ru = 0;
