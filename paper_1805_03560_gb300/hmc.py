@@ -173,8 +173,10 @@ def _lat_ref_of(L):
 
 def _lat_ref(L):
     """The lattice argument of a call.  Built once per lattice: making the
-    ctypes structure took 4 of the 16 us of an Mhat call on 8^3 x 16."""
-    return _lat_ref_of(tuple(L))
+    ctypes structure took 4 of the 16 us of an Mhat call on 8^3 x 16.  The key is
+    the extents as plain integers: zero-dimensional arrays have no hash, and
+    tensors hash by identity, whatever they hold by then."""
+    return _lat_ref_of(tuple(map(int, L)))
 
 
 def _ref(x):
