@@ -8,6 +8,7 @@ CPU fallback.
 import ctypes
 import functools
 import os
+import struct
 
 import numpy as np
 
@@ -166,17 +167,23 @@ def lattice(L):
     return Lat((ctypes.c_int * 4)(*[int(v) for v in L]))
 
 
+_pack_extents = struct.Struct("4i").pack
+
+
 @functools.lru_cache(maxsize=64)
-def _lat_ref_of(L):
-    return ctypes.byref(lattice(L))
+def _lat_ref_of(extents):
+    return ctypes.byref(Lat.from_buffer_copy(extents))
 
 
 def _lat_ref(L):
     """The lattice argument of a call.  Built once per lattice: making the
     ctypes structure took 4 of the 16 us of an Mhat call on 8^3 x 16.  The key is
-    the extents as plain integers: zero-dimensional arrays have no hash, and
-    tensors hash by identity, whatever they hold by then."""
-    return _lat_ref_of(tuple(map(int, L)))
+    the four integers' bytes: a zero-dimensional array has no hash, and a tensor
+    hashes by identity, whatever it holds by then."""
+    try:
+        return _lat_ref_of(_pack_extents(*L))
+    except struct.error:  # not four integers: lattice() converts or raises
+        return ctypes.byref(lattice(L))
 
 
 def _ref(x):

@@ -29,3 +29,11 @@ def test_extents_changed_in_place(H):
     assert _sites(H, L) == 960
     L[0].fill_(16)
     assert _sites(H, L) == 1920
+
+
+def test_other_numbers_and_counts(H):
+    """Whole floats convert and missing extents are zero (an invalid lattice), as lattice() has it."""
+    assert _sites(H, (8.0, 4.0, 6, 10)) == 960
+    assert _sites(H, (8, 4, 6)) == 0
+    with pytest.raises(IndexError):
+        _sites(H, (8, 4, 6, 10, 2))
