@@ -711,9 +711,19 @@ int dslash(hmc_ctx *ctx, const DslashArgs &a, const hmc_gauge &U, int sprec, int
                   a.n_rhs, a.mr_force);
     var = 2 + a.mr_force;
   }
-  if (a.cg_x && a.n_rhs > 1 && !(var >= 4 && var < 7))
+  // what the chosen kernel does not do is refused, not left out
+  const bool multi = var >= 4 && var < 7;
+  if (a.cg_x && !multi)
     return fail(ctx, HMC_EINVAL, "dslash: the fused batched update needs the multi-rhs kernel");
-  if (var >= 4 && var < 7 && nblocks)
+  if (multi && (a.red_src || (a.cg_r && !a.cg_x)))
+    return fail(ctx, HMC_EINVAL, "dslash: the multi-rhs kernel has neither the reduction block "
+                                 "nor the update of one system");
+  if (a.red_src && a.total)
+    return fail(ctx, HMC_EINVAL, "dslash: totals count the blocks of the launch, the reduction "
+                                 "block among them");
+  if (sprec == HMC_F64E && (a.partials || a.total || a.red_src || a.cg_r))
+    return fail(ctx, HMC_EINVAL, "dslash: emulated FP64 has no reductions and no fused update");
+  if (multi && nblocks)
     *nblocks = blocks_for((long long)a.g.Vh * (a.n_rhs / (var - 2)), DS_NT);
   DslashArgs la = a;
   la.pdl = ctx->pdl;

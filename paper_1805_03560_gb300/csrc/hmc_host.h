@@ -171,7 +171,9 @@ struct DslashArgs {
   double *total;
   unsigned int *counter;
   // one more block sums red_src[0..red_n) (the block partials a previous
-  // launch left) in a fixed order into *red_dst
+  // launch left) in a fixed order into *red_dst.  Refused together with total,
+  // by the multi-right-hand-side kernel and, like partials and cg_r, in
+  // emulated FP64
   const double *red_src;
   int red_n;
   double *red_dst;
