@@ -699,7 +699,7 @@ int dslash(hmc_ctx *ctx, const DslashArgs &a, const hmc_gauge &U, int sprec, int
   // -2: autotuned per class.
   int var = ctx->ds_variant >= 0 ? ctx->ds_variant : default_variant(ctx, U.fmt, sprec, a.n_rhs, nb);
   // small lattices: one thread per direction, unless a variant is asked for
-  const bool split = ctx->ds_variant < 0 && dslash_split_rule(ctx, a, sprec);
+  const bool split = ctx->ds_variant < 0 && dslash_split_rule(ctx, a, sprec, U.fmt);
   if (ctx->ds_variant == -2 && !split) var = tune_variant(ctx, a, sprec, U.fmt, dagger, nb);
   if (var >= 4 && var < 7 && !dslash_mr_supported(sprec, a.n_rhs, var - 2))
     var = U.fmt == 18 ? 2 : 0;

@@ -15,11 +15,12 @@
 // every SM has work from 4864 sites on, and inside a solve the loads of the
 // links, which none of its launches writes, are issued before the wait for
 // the launch before (links_ready).  Measured (one thread per site -> this
-// kernel): a CG iteration in FP32 on 8^3 x 16 33.1 -> 23.2 us, on 14 x 6 x 10
-// x 20 33.7 -> 24.8 us, on 12^3 x 24 36.8 -> 30.8 us; in FP64 155 -> 84, 201 ->
-// 131 and 282 -> 208 us; the emulated-FP64 hop 22.0 -> 9.7, 22.8 -> 10.8 and 30.4
-// -> 18.2 us (16.1 in the paired arithmetic).  (One thread per hop, eight warps to 32 sites, was slower for
-// FP32: 38.6 us per iteration on 12^3 x 24, the barrier's traffic doubles.)
+// kernel) on 8^3 x 16, 14 x 6 x 10 x 20 and 12^3 x 24: a CG iteration in FP32
+// 29.7 -> 20.5, 30.0 -> 23.0 and 35.8 -> 28.0 us, in FP64 156 -> 58, 183 -> 96 and
+// 286 -> 198 us; the emulated-FP64 hop 16.4 -> 9.0, 17.6 -> 10.3 and 30.6 -> 15.4 us.
+// (One thread per hop, eight warps to 32 sites, was slower for FP32: 38.6 us per
+// iteration on 12^3 x 24 against 36.8 with one thread per site then; the
+// barrier's traffic doubles.)
 #include "dslash_ops.cuh"
 #include "hmc_host.h"
 
@@ -286,21 +287,30 @@ int dslash_split_blocks(const Geo &g) { return blocks_for(g.Vh, SPLIT_SITES); }
 
 // The sites of the fullest SM decide: 32-site blocks spread the lattice
 // finer than 128-site blocks, at a cost per site (coordinates four times, the
-// exchange).  Measured, one thread per site against this kernel:
-//   FP32, per CG iteration: Vh 20736 36.8 / 30.8 us, 36864 40.4 / 39.2, 65536
-//     52.8 / 53.0, 81920 56.6 / 66.0: up to 256 sites per SM.
-//   emulated FP64, per hop: 20736 33.0 / 16.1 us, 36864 33.3 / 24.4, 65536
-//     41.6 / 45.7, 81920 50.2 / 50.3: up to 384 sites per SM.
-//   FP64 (bound by its pipe, 25 % dearer per site here), per CG iteration:
-//     20736 282 / 208 us, 36864 285 / 319, 65536 550 / 549, 128000 953 / 1034:
-//     where the fullest SM gets enough fewer sites.
-// Per-right-hand-side factors belong to several right-hand sides.
-bool dslash_split_rule(const hmc_ctx *ctx, const DslashArgs &a, int sprec) {
+// exchange).  Measured on 152 SMs, this kernel / one thread per site (the
+// default variant), by sites per parity:
+//   FP32, 12-real links, per CG iteration: 20736 28.0 / 35.8 us, 24192 28.1 /
+//     35.2 (the last size in one wave of five blocks per SM), 24576 33.0 / 35.2,
+//     28672 37.3 / 38.1, 31104 36.3 / 36.7, 34560 37.3 / 36.9, 38016 38.2 /
+//     36.2: up to 208 sites per SM, in the second wave until the two meet.
+//   FP32, 18-real links: 20736 30.3 / 35.9, 24192 30.4 / 35.1, 24576 35.5 / 35.2,
+//     27648 38.2 / 36.7, 36864 41.5 / 37.3: up to 160 sites per SM, one wave.
+//   emulated FP64, 18-real links, per hop: 20736 15.4 / 30.6, 40960 26.3 / 31.2,
+//     49152 31.3 / 31.7, 55296 35.5 / 31.9: up to 320 sites per SM.
+//   emulated FP64, 12-real links, per hop: 20736 18.1 / 36.0, 40960 29.6 / 38.2,
+//     57344 40.5 / 42.2: up to 384 sites per SM, one wave of the other kernel.
+//   FP64, per CG iteration: 20736 198 / 286, 24576 231 / 287, 34560 302 / 290,
+//     40960 338 / 421, 55296 440 / 422: where the fullest SM gets a fifth fewer
+//     sites (the cost per site is 4 to 6 % higher here; with fewer than a fifth
+//     the gain is 4 to 8 %: 49152 407 / 424, 65536 514 / 553).
+// Half storage has no form of this kernel.  Per-right-hand-side factors belong to
+// several right-hand sides.
+bool dslash_split_rule(const hmc_ctx *ctx, const DslashArgs &a, int sprec, int fmt) {
   if (a.n_rhs != 1 || a.cb_rhs) return false;
   const long long Vh = a.g.Vh, sms = ctx->sm_count;
   switch (sprec) {
-    case HMC_F32: return Vh <= 256 * sms;
-    case HMC_F64E: return Vh <= 384 * sms;
+    case HMC_F32: return Vh <= (fmt == 18 ? 160 : 208) * sms;
+    case HMC_F64E: return Vh <= (fmt == 18 ? 320 : 384) * sms;
     case HMC_F64: {
       const long long fine = (Vh + SPLIT_SITES * sms - 1) / (SPLIT_SITES * sms) * SPLIT_SITES;
       const long long coarse = (Vh + DS_NT * sms - 1) / (DS_NT * sms) * DS_NT;

@@ -228,7 +228,7 @@ void launch_dslash_e2(DslashArgs a, int dagger, cudaStream_t st);
 // One-thread-per-direction hemi-Dslash (dslash_split.cu) of one right-hand
 // side: whether it is the kernel for this launch, its launch, and its block
 // count (the partials it leaves; the kernels of DS_NT threads leave fewer).
-bool dslash_split_rule(const hmc_ctx *ctx, const DslashArgs &a, int sprec);
+bool dslash_split_rule(const hmc_ctx *ctx, const DslashArgs &a, int sprec, int fmt);
 bool launch_dslash_split(const hmc_ctx *ctx, const DslashArgs &a, int sprec, int fmt, int dagger);
 int dslash_split_blocks(const Geo &g);
 // Multi-right-hand-side hemi-Dslash with nr right-hand sides per thread

@@ -1,0 +1,46 @@
+"""The rule that gives a launch to the one-thread-per-direction hemi-Dslash
+takes none that measured slower there (by more than 3 %) on a GPU of 152 SMs,
+and takes those that gain 15 % or more: microseconds per CG iteration (FP32,
+FP64) or per hemi-Dslash (emulated FP64), one thread per direction / one thread
+per site."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+F64, F32, F64E = 0, 1, 3
+# (precision, link format): {sites per parity: (per direction, per site)}
+MEASURED = {
+    (F32, 12): {4096: (20.5, 29.7), 20736: (28.0, 35.8), 24576: (33.0, 35.2), 38016: (38.2, 36.2),
+                49152: (47.2, 41.7)},
+    (F32, 18): {4096: (21.4, 28.5), 20736: (30.3, 35.9), 24192: (30.4, 35.1), 27648: (38.2, 36.7),
+                36864: (41.5, 37.3)},
+    (F64, 18): {4096: (58.3, 156.5), 24576: (230.8, 286.5), 34560: (302.2, 289.5),
+                40960: (338.1, 420.9), 55296: (439.6, 422.1)},
+    (F64E, 18): {4096: (9.0, 16.4), 24576: (17.2, 28.1), 40960: (26.3, 31.2), 55296: (35.5, 31.9),
+                 57344: (36.7, 32.3)},
+    (F64E, 12): {4096: (10.4, 28.3), 40960: (29.6, 38.2), 57344: (40.5, 42.2)},
+}
+POINTS = [(p, f, Vh, t) for (p, f), m in MEASURED.items() for Vh, t in m.items()]
+
+
+@pytest.fixture(scope="module")
+def taken(tmp_path_factory):
+    from paper_1805_03560_gb300 import build as B
+    B.build()
+    exe = str(tmp_path_factory.mktemp("rule") / "split_rule")
+    subprocess.run([B.nvcc(), *B.ARCH, *B.FLAGS, "-I", B.CSRC,
+                    os.path.join(ROOT, "tests", "c_client", "split_rule.cu"),
+                    "-L", B.HERE, "-lhmc", "-Xlinker", "-rpath", "-Xlinker", B.HERE, "-o", exe],
+                   check=True)
+    args = [str(v) for p in POINTS for v in p[:3]]
+    out = subprocess.run([exe, *args], check=True, capture_output=True, text=True).stdout
+    return [int(v) for v in out.split()]
+
+
+def test_rule_against_measured_times(taken):
+    assert len(taken) == len(POINTS)
+    wrong = [q for q, on in zip(POINTS, taken)
+             if on and q[3][0] > 1.03 * q[3][1] or not on and 1.15 * q[3][0] < q[3][1]]
+    assert not wrong, wrong
