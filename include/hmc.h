@@ -155,7 +155,7 @@ int hmc_ctx_set_timing(hmc_ctx *ctx, int enable);
  * 1; otherwise consecutive sites), bit 1 issues the loads of both hops of a
  * direction before their arithmetic (for F16/BF16 storage with 12-real links:
  * of the four hops of two directions).  Variants 0..3 compute the same result
- * bit for bit.  Values 4, 5, 6 select, for n_rhs > 1 and FP32 or FP16 storage,
+ * bit for bit (in emulated FP64 with LINK18 they are one kernel).  Values 4, 5, 6 select, for n_rhs > 1 and FP32 or FP16 storage,
  * the multi-right-hand-side kernel with 2, 3 or 4 right-hand sides per thread
  * (each link loaded, rebuilt and indexed once for them, packed paired-FP32
  * arithmetic; exact on exactly representable inputs, otherwise within FP32
@@ -170,11 +170,12 @@ int hmc_ctx_set_timing(hmc_ctx *ctx, int enable);
  * fill the GPU better (by the lattice size).  With -1 and -2, one right-hand
  * side in FP64, FP32 or emulated FP64 on a lattice too small to fill the GPU
  * runs one thread per site and direction (the four directions' sums added last:
- * within rounding of the other variants).  -2: autotune: the first launch of
- * each class (precision, link format, dagger, n_rhs, lattice) that can be repeated without
- * changing its result times every applicable variant (one warm-up and three
- * timed launches each, synchronising the stream) and the class keeps the
- * fastest; the solvers tune their classes on scratch fields before iterating.
+ * within rounding of the other variants).  -2: autotune: elsewhere the first
+ * launch of each class (precision, link format, dagger, n_rhs, lattice) that can
+ * be repeated without changing its result times every applicable variant (one
+ * warm-up and three timed launches each, synchronising the stream) and the
+ * class keeps the fastest; the solvers tune their classes on scratch fields
+ * before iterating.  For one right-hand side -2 gives the bits of -1.
  * Launches during stream capture are never tuned. */
 #define HMC_OPT_DSLASH_VARIANT 1
 /* HMC_OPT_CG_GRAPH: 1 (default) runs every CG solve of hmc_cg_solve and

@@ -527,7 +527,10 @@ static bool launch_variant(const DslashArgs &a, int sprec, int fmt, int dagger, 
 // stream, which it synchronises) and keeps the fastest for the class; every
 // later launch of the class, with or without an epilogue, uses it.  Launches
 // of an untuned class that cannot be repeated, and launches while the stream
-// is being captured, use the built-in default.
+// is being captured, use the built-in default.  The one-thread-per-direction
+// kernel is not timed against them: it sums the directions in another order,
+// and a choice by timing would make the bits of a solve depend on it, so there
+// dslash_split_rule decides alone, for the default as for this mode.
 static std::string tune_key(const DslashArgs &a, int sprec, int fmt, int dagger) {
   char k[96];
   snprintf(k, sizeof k, "%d/%d/%d/%d/%d.%d.%d.%d", sprec, fmt, dagger, a.n_rhs, a.g.L[0], a.g.L[1],
@@ -605,6 +608,9 @@ static bool launch_any(const DslashArgs &a, int sprec, int fmt, int dagger, int 
   return launch_variant(a, sprec, fmt, dagger, v, nb, st);
 }
 
+// variants 0..3 of emulated FP64 with 18-real links are one kernel (dslash_e2.cu)
+static bool one_variant(int sprec, int fmt) { return sprec == HMC_F64E && fmt == 18; }
+
 static int tune_variant(hmc_ctx *ctx, const DslashArgs &a, int sprec, int fmt, int dagger, int nb) {
   const std::string key = tune_key(a, sprec, fmt, dagger);
   auto it = ctx->ds_tuned.find(key);
@@ -614,6 +620,7 @@ static int tune_variant(hmc_ctx *ctx, const DslashArgs &a, int sprec, int fmt, i
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(ctx->stream, &cs);
   const int dflt = default_variant(ctx, fmt, sprec, a.n_rhs, nb);
+  if (one_variant(sprec, fmt)) return dflt;
   if (!repeatable || cs != cudaStreamCaptureStatusNone || ctx->tune_frozen) return dflt;
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess) return dflt;
@@ -745,12 +752,24 @@ int dslash(hmc_ctx *ctx, const DslashArgs &a, const hmc_gauge &U, int sprec, int
   return launched(ctx, cls);
 }
 
+// Whether the launches to come of (sprec, U.fmt, n_rhs, cb_rhs) have variants to
+// tune: the context autotunes, there is more than one, and they do not run one
+// thread per direction.
+bool dslash_tunes(const hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, int sprec, int n_rhs,
+                  const double *cb_rhs) {
+  DslashArgs a{};
+  a.g = g;
+  a.n_rhs = n_rhs;
+  a.cb_rhs = cb_rhs;
+  return ctx->ds_variant == -2 && U.prec == sprec && !one_variant(sprec, U.fmt) &&
+         !dslash_split_rule(ctx, a, sprec, U.fmt);
+}
+
 // Tune the variant classes of (sprec, U.fmt, n_rhs) for both daggers on
-// scratch fields: out is overwritten, in only read (no-op unless the context
-// autotunes).
+// scratch fields: out is overwritten, in only read (no-op unless dslash_tunes).
 int dslash_tune(hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, int sprec, int n_rhs, void *out,
-                const void *in) {
-  if (ctx->ds_variant != -2 || U.prec != sprec) return HMC_OK;
+                const void *in, const double *cb_rhs) {
+  if (!dslash_tunes(ctx, g, U, sprec, n_rhs, cb_rhs)) return HMC_OK;
   DslashArgs a{};
   a.g = g;
   a.n_rhs = n_rhs;

@@ -56,14 +56,15 @@ int hi_mhat(const HiOps &h, int dagger, void *out, const void *in, double kappa,
 // scratch fields (no allocation may happen while a stream is captured) and,
 // in autotuning contexts, tune their hemi-Dslash classes on scratch (zeroed
 // input), so that the captured launches use the tuned variants.
-int hi_prepare(const HiOps &h, int n_rhs) {
+int hi_prepare(const HiOps &h, int n_rhs, const double *cb_rhs) {
   void *in = hi_ws(h, "in", n_rhs), *out = hi_ws(h, "out", n_rhs);
   void *tmp = hi_ws(h, "tmp", n_rhs), *mid = hi_ws(h, "mid", n_rhs);
   if (!in || !out || !tmp || !mid) return HMC_ENOMEM;
-  if (h.ctx->ds_variant != -2) return HMC_OK;
   const int p = h.emul ? HMC_F64E : HMC_F64;
+  const hmc_gauge &U = h.emul ? h.Ue : h.Uh;
+  if (!dslash_tunes(h.ctx, h.g, U, p, n_rhs, cb_rhs)) return HMC_OK;
   TRY(zero_field(h.ctx, p, in, h.g.Vh * n_rhs));
-  return dslash_tune(h.ctx, h.g, h.emul ? h.Ue : h.Uh, p, n_rhs, tmp, in);
+  return dslash_tune(h.ctx, h.g, U, p, n_rhs, tmp, in, cb_rhs);
 }
 
 // out = Mhat^dag Mhat in

@@ -41,8 +41,8 @@ struct hmc_ctx {
   // the time since the previous event to that launch (a launch timeline).
   int timing = 0;
   cudaEvent_t trace_prev = nullptr;
-  // hemi-Dslash kernel variant: bit 0 tiled site mapping, bit 1 paired loads;
-  // -1 chooses per link format
+  // hemi-Dslash kernel variant (HMC_OPT_DSLASH_VARIANT): -1 chooses by precision,
+  // link format, right-hand sides and lattice size
   int ds_variant = -1;
   int ds_rev = 0;    // direction of the last hemi-Dslash launch (DslashArgs::rev)
   int sm_count = 1;  // streaming multiprocessors of the device
@@ -241,10 +241,12 @@ bool launch_dslash_mr(const DslashArgs &a, int sprec, int fmt, int dagger, int n
 int dslash_mr_nr(hmc_ctx *ctx, const Geo &g, int sprec, int fmt, int n_rhs);
 int dslash(hmc_ctx *ctx, const DslashArgs &a, const hmc_gauge &U, int sprec, int dagger,
            int *nblocks);
+bool dslash_tunes(const hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, int sprec, int n_rhs,
+                  const double *cb_rhs);
 // autotune the hemi-Dslash classes of (sprec, U.fmt, n_rhs) on scratch fields
-// (no-op unless HMC_OPT_DSLASH_VARIANT is -2)
+// (no-op unless dslash_tunes; cb_rhs: as in the launches to come)
 int dslash_tune(hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, int sprec, int n_rhs, void *out,
-                const void *in);
+                const void *in, const double *cb_rhs = nullptr);
 
 // n complex numbers of 16 bytes, F64 -> F64E
 void chunks_to_f64e(hmc_ctx *ctx, void *dst, const void *src, long long n);
@@ -374,7 +376,7 @@ int hi_begin(hmc_ctx *ctx, const Geo &g, const hmc_gauge &Uh, const hmc_solver_o
              HiOps *h, const char *tag);
 // F64 fields in and out; n_rhs right-hand sides with per-RHS -kappa^2 in
 // cb_rhs (device, nullable)
-int hi_prepare(const HiOps &h, int n_rhs = 1);
+int hi_prepare(const HiOps &h, int n_rhs = 1, const double *cb_rhs = nullptr);
 int hi_mhat(const HiOps &h, int dagger, void *out, const void *in, double kappa, int n_rhs,
             const double *cb_rhs);
 int hi_mdagm(const HiOps &h, void *out, const void *in, double kappa, int n_rhs,

@@ -603,12 +603,12 @@ int cg_solve_multi(hmc_ctx *ctx, const Geo &g, const hmc_gauge &Uh, const hmc_ga
   // scratch (t = H p); the fused last hop then runs the multi-right-hand-side
   // kernel with the tuned (or default) right-hand sides per thread
   if (mixed) {
-    TRY(dslash_tune(ctx, g, s.Ul, s.plo, n_rhs, s.tlo, s.p));
+    TRY(dslash_tune(ctx, g, s.Ul, s.plo, n_rhs, s.tlo, s.p, s.cb));
     s.mr = dslash_mr_nr(ctx, g, s.plo, s.Ul.fmt, n_rhs);
   }
   s.tol2 = tol * tol;
   // the FP64-accurate operator's scratch (and tuned classes) for the capture
-  TRY(hi_prepare(s.hi, n_rhs));
+  TRY(hi_prepare(s.hi, n_rhs, s.cb));
   const int cap = max_iter > 0 ? max_iter : 0;
   const long long bodies = 2LL * cap + 16;
   k_mcontrol_init<<<1, 1, 0, ctx->stream>>>(s.st, n_rhs, delta * delta, cap, mixed ? 1 : 0,
