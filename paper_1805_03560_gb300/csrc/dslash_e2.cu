@@ -32,12 +32,9 @@ __global__ void __launch_bounds__(DS_NT, 3) k_dslash_e2(const DslashArgs a) {
   if (a.gate && *a.gate == 0) return;
   const int Vh = a.g.Vh, S_ = Vh * a.n_rhs;
   const int blk = ds_block(a, blockIdx.x), i = blk * DS_NT + threadIdx.x;
-  double nrm = 0.0;
-  int r_out = -1;
   if (i < S_) {
     const int h = a.n_rhs == 1 ? i : i / a.n_rhs;
     const int r = i - h * a.n_rhs;
-    r_out = r;
     int c[4];
     const int lex = site_coords(a.g, h, a.p, c);
     float4 *slot = s_buf + threadIdx.x;  // slot k at slot[k * DS_NT]
@@ -95,22 +92,6 @@ __global__ void __launch_bounds__(DS_NT, 3) k_dslash_e2(const DslashArgs a) {
       for (int k = 0; k < 12; ++k) acc[k] = cb * acc[k];
     }
     SIO::store(a.out, S_, i, acc);
-    if (a.partials) {
-      R n2 = R(0);
-#pragma unroll
-      for (int k = 0; k < 12; ++k) n2 += norm2(acc[k]);
-      nrm = (double)n2;
-    }
-  }
-  if (a.partials) {
-    if (a.n_rhs == 1) {
-      const double t = block_sum<DS_NT>(nrm);
-      if (threadIdx.x == 0) a.partials[blk] = t;
-      if (a.total) last_block_total<DS_NT>(a.partials, a.counter, a.total);
-    } else {
-      block_partials_rhs<DS_NT>(nrm, r_out, a.n_rhs, a.partials);
-      if (a.total) last_block_totals_rhs<DS_NT>(a.partials, a.n_rhs, a.counter, a.total);
-    }
   }
 }
 

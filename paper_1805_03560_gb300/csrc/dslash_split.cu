@@ -253,7 +253,6 @@ __global__ void __launch_bounds__(SPLIT_NT, split_min_blocks<SP>()) k_dslash_spl
       for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
       if (lane == 0) a.partials[blockIdx.x] = s;
     }
-    if (a.total) last_block_total<SPLIT_NT>(a.partials, a.counter, a.total);
   }
 }
 
@@ -303,10 +302,10 @@ int dslash_split_blocks(const Geo &g) { return blocks_for(g.Vh, SPLIT_SITES); }
 //     40960 338 / 421, 55296 440 / 422: where the fullest SM gets a fifth fewer
 //     sites (the cost per site is 4 to 6 % higher here; with fewer than a fifth
 //     the gain is 4 to 8 %: 49152 407 / 424, 65536 514 / 553).
-// Half storage has no form of this kernel.  Per-right-hand-side factors belong to
-// several right-hand sides.
+// Half storage has no form of this kernel.  Per-right-hand-side factors and totals
+// (the batched CG's) are not part of it.
 bool dslash_split_rule(const hmc_ctx *ctx, const DslashArgs &a, int sprec, int fmt) {
-  if (a.n_rhs != 1 || a.cb_rhs) return false;
+  if (a.n_rhs != 1 || a.cb_rhs || a.total) return false;
   const long long Vh = a.g.Vh, sms = ctx->sm_count;
   switch (sprec) {
     case HMC_F32: return Vh <= (fmt == 18 ? 160 : 208) * sms;

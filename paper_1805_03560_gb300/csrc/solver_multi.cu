@@ -548,7 +548,7 @@ int cg_solve_multi(hmc_ctx *ctx, const Geo &g, const hmc_gauge &Uh, const hmc_ga
   const double delta = (opts && opts->reliable_delta > 0) ? opts->reliable_delta : 0.1;
   const int check = (opts && opts->check_every > 0) ? opts->check_every : 16;
   s.S = g.Vh * n_rhs;
-  s.nb_ds = n_rhs == 1 ? dslash_split_blocks(g) : blocks_for(s.S, DS_NT);
+  s.nb_ds = blocks_for(s.S, DS_NT);
   s.nb_bl = blocks_for(s.S, BL_NT);
   const size_t f64 = spinor_bytes(g, HMC_F64, n_rhs);
   s.st = (MState *)workspace(ctx, "cgm_state", sizeof(MState));
