@@ -275,7 +275,7 @@ int hop_force_multi(hmc_ctx *ctx, const Geo &g, const hmc_gauge &U, int n, const
     case HMC_F64 * 100 + 12: k_hop_force<12, HMC_F64><<<nb, HF_NT, 0, st>>>(a); break;
     case HMC_F32 * 100 + 18: k_hop_force<18, HMC_F32><<<nb, HF_NT, 0, st>>>(a); break;
     case HMC_F32 * 100 + 12: k_hop_force<12, HMC_F32><<<nb, HF_NT, 0, st>>>(a); break;
-    // emulated FP64: the outer products and Q = U A - B U^dag in double-float
+    // emulated FP64: the outer products and U (A + B^dag) in double-float
     case HMC_F64E * 100 + 18: launch_hop_force_e2<18>(a, nb, st); break;
     case HMC_F64E * 100 + 12: launch_hop_force_e2<12>(a, nb, st); break;
     default: return fail(ctx, HMC_EINVAL, "force: bad link format %d", U.fmt);

@@ -39,9 +39,9 @@ struct CGState {
   double rr[2];   // |r|^2 at the start of iteration k is rr[k & 1]
   double b2, tol2;
   double aux;     // scratch for one-off reductions
-  double pap;     // p^dag A p of the current iteration (last block of the Mhat Dslash)
+  double pap;     // p^dag A p of the current iteration (extra block of the H_eo^dag launch)
   double rr_next; // |r|^2 after the update (set by xpay)
-  double alpha;   // rr / pap of the current iteration (block 0 of the H_eo^dag launch)
+  double alpha;   // rr / pap of the current iteration (the same block)
   int done;       // 1 converged (recursive residual), 2 NaN/Inf
   // gate[par]: the launches of an iteration of parity par run; xpay of parity
   // par sets the other one (it may stop the solve while blocks of its own
@@ -686,7 +686,7 @@ int one_iteration(Solve &s, int k, const Handles &h = Handles()) {
   int nb_pap = 0;
   TRY(dslash(ctx, a, U, s.plo, 0, &nb_pap));
   a.partials = nullptr;
-  // t = H_eo^dag y, block 0 finishing p^dag A p
+  // t = H_eo^dag y, an extra block finishing p^dag A p
   a.p = 1; a.out = s.tlo; a.in = s.y; a.x = nullptr; a.ca = 0.0; a.cb = 1.0;
   a.red_src = s.pap_part; a.red_n = nb_pap; a.red_dst = &s.st->pap;
   a.red_rr = &s.st->rr[par]; a.red_alpha = &s.st->alpha; a.red_flag = &s.st->done;
