@@ -3,14 +3,16 @@
 // arithmetic of df64x2.cuh.
 //
 // What bounds it is the FP32 pipe: about 700 paired operations (two pipe
-// cycles each) per hop, 103 of the 158 us of a hop on 24^3 x 48; three-register
-// operands and register banks keep the pipe from more than about two thirds
+// cycles each) per hop, 103 of the 139 us of a hop on 24^3 x 48; three-register
+// operands and register banks keep the pipe from more than about three quarters
 // (sixteen warps per SM in 128 registers: 164 us, twelve: 160).  The eight hops
 // run in a loop, and while one is computed the next hop's spinor and link come
 // into the thread's own slots of shared memory (cp.async; the links in two
 // buffers, the spinor's slots are free once it is projected), 165 -> 160 us.  No
 // barrier: every thread reads what it asked for itself.  Measured against the
-// scalar double-float form: 24^3 x 48 184 -> 160 us, 32^3 x 64 567 -> 477 us.
+// scalar double-float form: 24^3 x 48 184 -> 160 us, 32^3 x 64 567 -> 477 us.  Without
+// the reductions of dslash.cu, which nothing asks for in this precision (4 KB of
+// shared memory, six registers), 159 -> 139 us and 406 us.
 #include "dslash_ops.cuh"
 #include "hmc_host.h"
 

@@ -17,7 +17,7 @@
 // the launch before (links_ready).  Measured (one thread per site -> this
 // kernel) on 8^3 x 16, 14 x 6 x 10 x 20 and 12^3 x 24: a CG iteration in FP32
 // 29.7 -> 20.5, 30.0 -> 23.0 and 35.8 -> 28.0 us, in FP64 156 -> 58, 183 -> 96 and
-// 286 -> 198 us; the emulated-FP64 hop 16.4 -> 9.0, 17.6 -> 10.3 and 30.6 -> 15.4 us.
+// 286 -> 198 us; the emulated-FP64 hop 14.1 -> 9.0, 16.9 -> 10.0 and 26.5 -> 15.1 us.
 // (One thread per hop, eight warps to 32 sites, was slower for FP32: 38.6 us per
 // iteration on 12^3 x 24 against 36.8 with one thread per site then; the
 // barrier's traffic doubles.)
@@ -294,8 +294,9 @@ int dslash_split_blocks(const Geo &g) { return blocks_for(g.Vh, SPLIT_SITES); }
 //     36.2: up to 208 sites per SM, in the second wave until the two meet.
 //   FP32, 18-real links: 20736 30.3 / 35.9, 24192 30.4 / 35.1, 24576 35.5 / 35.2,
 //     27648 38.2 / 36.7, 36864 41.5 / 37.3: up to 160 sites per SM, one wave.
-//   emulated FP64, 18-real links, per hop: 20736 15.4 / 30.6, 40960 26.3 / 31.2,
-//     49152 31.3 / 31.7, 55296 35.5 / 31.9: up to 320 sites per SM.
+//   emulated FP64, 18-real links, per hop: 20736 15.1 / 26.5, 40960 26.0 / 27.9,
+//     42336 26.7 / 28.5, 44352 29.0 / 28.5, 49152 31.2 / 27.6: up to 288 sites per
+//     SM, three waves of three blocks.
 //   emulated FP64, 12-real links, per hop: 20736 18.1 / 36.0, 40960 29.6 / 38.2,
 //     57344 40.5 / 42.2: up to 384 sites per SM, one wave of the other kernel.
 //   FP64, per CG iteration: 20736 198 / 286, 24576 231 / 287, 34560 302 / 290,
@@ -309,7 +310,7 @@ bool dslash_split_rule(const hmc_ctx *ctx, const DslashArgs &a, int sprec, int f
   const long long Vh = a.g.Vh, sms = ctx->sm_count;
   switch (sprec) {
     case HMC_F32: return Vh <= (fmt == 18 ? 160 : 208) * sms;
-    case HMC_F64E: return Vh <= (fmt == 18 ? 320 : 384) * sms;
+    case HMC_F64E: return Vh <= (fmt == 18 ? 288 : 384) * sms;
     case HMC_F64: {
       const long long fine = (Vh + SPLIT_SITES * sms - 1) / (SPLIT_SITES * sms) * SPLIT_SITES;
       const long long coarse = (Vh + DS_NT * sms - 1) / (DS_NT * sms) * DS_NT;

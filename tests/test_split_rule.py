@@ -18,8 +18,8 @@ MEASURED = {
                 36864: (41.5, 37.3)},
     (F64, 18): {4096: (58.3, 156.5), 24576: (230.8, 286.5), 34560: (302.2, 289.5),
                 40960: (338.1, 420.9), 55296: (439.6, 422.1)},
-    (F64E, 18): {4096: (9.0, 16.4), 24576: (17.2, 28.1), 40960: (26.3, 31.2), 55296: (35.5, 31.9),
-                 57344: (36.7, 32.3)},
+    (F64E, 18): {4096: (9.0, 14.1), 24576: (17.1, 26.7), 42336: (26.7, 28.5), 45056: (29.8, 27.8),
+                 57344: (36.6, 28.1)},
     (F64E, 12): {4096: (10.4, 28.3), 40960: (29.6, 38.2), 57344: (40.5, 42.2)},
 }
 POINTS = [(p, f, Vh, t) for (p, f), m in MEASURED.items() for Vh, t in m.items()]
