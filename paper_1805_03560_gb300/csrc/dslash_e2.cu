@@ -12,7 +12,7 @@
 // barrier: every thread reads what it asked for itself.  Measured against the
 // scalar double-float form: 24^3 x 48 184 -> 160 us, 32^3 x 64 567 -> 477 us.  Without
 // the reductions of dslash.cu, which nothing asks for in this precision (4 KB of
-// shared memory, six registers), 159 -> 139 us and 406 us.
+// shared memory, six registers), 158 -> 139 us and 406 us.
 #include "dslash_ops.cuh"
 #include "hmc_host.h"
 

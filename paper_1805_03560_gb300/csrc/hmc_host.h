@@ -214,9 +214,11 @@ struct DslashArgs {
 // lattice larger than L2 a launch that walks the same way as the one before
 // finds everything evicted, one that walks the other way starts on what was
 // touched last.  Measured (all launches the same way -> alternating): Mhat in
-// FP32 on 24^3 x 48 72.0 -> 64.8 us, a CG iteration there 201.9 -> 187.7 us in
-// FP32 and 174.3 -> 166.8 us in F16, on 32^3 x 64 582.9 -> 563.4 us; no
-// difference where the fields fit in L2.  Results do not depend on it: a
+// FP32 on 24^3 x 48 70.5 -> 67.0 us, a CG iteration (its share of the reliable
+// updates included) there 192 -> 179 us in FP32 and 160 -> 153 us in F16, on
+// 32^3 x 64 555 -> 540 and 461 -> 451 us; no difference where the fields fit in
+// L2.  DRAM reads of the second to fourth hemi-Dslash of an iteration in FP32 on
+// 24^3 x 48: 190, 160, 224 -> 136, 118, 166 MB.  Results do not depend on it: a
 // block's partial sum is stored under the lattice block it belongs to.
 // b: the block's number among those that work on the lattice.
 __device__ __forceinline__ int ds_block(const DslashArgs &a, int b) {
